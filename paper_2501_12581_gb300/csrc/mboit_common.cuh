@@ -301,6 +301,9 @@ struct GenericBlend {
 // Bodies that take two lattice points at once (pair(...), equal to two calls).
 template <class B> struct HasPair : std::false_type {};
 template <> struct HasPair<GenericBlend> : std::true_type {};
+// Bodies that are told the unit (brick or tet) of every point before its
+// sample, and may decline it (bool enter(int unit)).
+template <class B> struct TakesUnits : std::false_type {};
 // Bodies whose per-sample code is short enough to copy into a fully
 // unrolled chunk loop (the four-power-moment blends).  The bodies of 6 and 8
 // power moments and of trigonometric moments (root solves, series) take the

@@ -251,7 +251,7 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
             const float tz = lattice_t(kz, g.step);
             store.seek(ka);
             float t0 = lattice_t(ka, g.step);
-            if constexpr (!kSel) {
+            if constexpr (!kSel && !TakesUnits<Body>::value) {
                 // two points at a time: both positions, then both points' 16
                 // window reads, then the store and the body in order
                 auto window_value = [&](float t) {
@@ -275,9 +275,11 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
             for (float t = t0; t <= tz; t += g.step) {
                 const float p0 = ffma(t, d[0], o[0]), p1 = ffma(t, d[1], o[1]), p2 = ffma(t, d[2], o[2]);
                 const int ix = (int)p0, iy = (int)p1, iz = (int)p2;
-                if (kSel) {
+                if (kSel || TakesUnits<Body>::value) {
                     const int b = ((iz >> g.brick_log2) * g.nby + (iy >> g.brick_log2)) * g.nbx + (ix >> g.brick_log2);
-                    if (!__ldg(sel + b)) {
+                    if constexpr (TakesUnits<Body>::value) {
+                        if (!body.enter(b)) continue;
+                    } else if (!__ldg(sel + b)) {
                         store.put(__int_as_float(0x7fc00000));
                         continue;
                     }
@@ -296,6 +298,12 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
             store.seek(ka);
             for (float t = lattice_t(ka, g.step); t <= tz; t += g.step) {
                 float val;
+                if constexpr (TakesUnits<Body>::value) {
+                    // every point of [k0, k1] is inside the domain
+                    const int ix = (int)ffma(t, d[0], o[0]), iy = (int)ffma(t, d[1], o[1]), iz = (int)ffma(t, d[2], o[2]);
+                    if (!body.enter(((iz >> g.brick_log2) * g.nby + (iy >> g.brick_log2)) * g.nbx + (ix >> g.brick_log2)))
+                        continue;
+                }
                 if (!field_sample<kSel>(g, sel, t, o, d, val)) {
                     store.put(__int_as_float(0x7fc00000));
                     continue;

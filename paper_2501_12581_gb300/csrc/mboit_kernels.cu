@@ -354,6 +354,7 @@ cudaError_t prepare_grid_kernels();
 cudaError_t prepare_frame_kernels();
 cudaError_t prepare_frame_unit_kernels();
 cudaError_t prepare_unit_kernels();
+cudaError_t prepare_piece_kernels();
 
 cudaError_t prepare_kernels() {
     // Loads every kernel and fills the occupancy cache, so that no module
@@ -375,6 +376,7 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess) e = prepare_multi_kernels();
     if (e == cudaSuccess) e = prepare_multi_amr_kernels();
     if (e == cudaSuccess) e = prepare_unit_kernels();
+    if (e == cudaSuccess) e = prepare_piece_kernels();
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -547,7 +547,9 @@ __device__ __forceinline__ void march_unit(const TetT<kNarrow>& m, const uint8_t
         }
         const bool found = f == -1 || tet_search<kNarrow>(m, w, q, D);
         float val = __int_as_float(0x7fc00000);
-        if (found && (!kSel || __ldg(sel + w.T))) {
+        bool take = found && (!kSel || __ldg(sel + w.T));
+        if constexpr (TakesUnits<Body>::value) take = take && body.enter(w.T);
+        if (take) {
             // the corner values (the .w words) read again here rather than
             // kept live through the walk, which only tests x, y, z: fewer
             // spilled registers in the loop (the same bits, so the same value)
