@@ -80,6 +80,7 @@ struct mboit_volume_s {
     int4* d_leaves = nullptr;
     float4* d_leaf_box = nullptr;
     int32_t* d_fmap = nullptr;
+    uint32_t* d_bricks = nullptr;
     std::vector<int32_t> leaf_table;
     mb::TetD tet{};             // tetrahedral meshes: amr-like parameters plus the device tables below
     int4* d_tcorners = nullptr;
@@ -1028,6 +1029,23 @@ mboit_status mboit_create_volume(const mboit_volume_desc* d, mboit_volume* out) 
         v->amr.max_level = d->max_level;
         v->amr.complete = std::find(fmap.begin(), fmap.end(), -1) == fmap.end() ? 1 : 0;
         v->amr.n_leaves = d->n_leaves;
+        // one word per finest brick for pass 1 (AmrD::bricks)
+        bool words = v->amr.complete && d->brick_log2 == 3 && d->n_leaves < (1 << mb::kBrickIdBits) &&
+                     (int64_t)d->n_leaves * 729 < INT32_MAX;
+        for (int32_t l = 0; words && l < d->n_leaves; ++l) {
+            const int32_t* L = d->leaf_table + 4 * (size_t)l;
+            const int32_t size = 8 << (d->max_level - L[3]);
+            words = L[0] % size == 0 && L[1] % size == 0 && L[2] % size == 0;
+        }
+        if (words) {
+            std::vector<uint32_t> w(fmap.size());
+            for (size_t i = 0; i < w.size(); ++i)
+                w[i] = mb::brick_word(fmap[i], d->max_level - d->leaf_table[4 * (size_t)fmap[i] + 3]);
+            if (e == cudaSuccess) e = cudaMalloc(&v->d_bricks, w.size() * sizeof(uint32_t));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(v->d_bricks, w.data(), w.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+            v->amr.bricks = v->d_bricks;
+        }
         v->amr.err = &v->d_ctr->error;
     }
     if (e == cudaSuccess && is_tet) {
@@ -1093,6 +1111,7 @@ mboit_status mboit_destroy_volume(mboit_volume v) {
         cudaFree(v->d_leaves);
         cudaFree(v->d_leaf_box);
         cudaFree(v->d_fmap);
+        cudaFree(v->d_bricks);
         cudaFree(v->d_tcorners);
         cudaFree(v->d_tnbrs);
         cudaFree(v->d_tcells);

@@ -135,6 +135,7 @@ __device__ __forceinline__ float trilinear8(float v000, float v100, float v010, 
 struct NoStore {
     __device__ __forceinline__ void seek(int) {}
     __device__ __forceinline__ void put(float) {}
+    __device__ __forceinline__ void skip() {}
 };
 struct RowStore {
     float* base;  // slot of row 0: vals + (tile_base - kmin) * 32 + lane; NULL: off
@@ -144,6 +145,7 @@ struct RowStore {
         if (base) __stcs(at, v);  // streaming store: read once by pass 2, keep the field in L2
         at += 32;
     }
+    __device__ __forceinline__ void skip() { at += 32; }
 };
 
 // Depth terms of lattice depth t for four power moments: the warped depth z

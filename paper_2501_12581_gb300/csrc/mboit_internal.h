@@ -81,8 +81,16 @@ struct AmrD {
     int32_t complete;       // 1: every finest brick has a leaf (no holes)
     int32_t n_leaves;       // leaf ids are 0 .. n_leaves - 1 (checked where the map is read)
     int32_t pad;
+    // Per finest brick its leaf and that leaf's 1 / cell size in one word (the
+    // leaf id in the mantissa of the power of two, brick_word), or NULL: octrees
+    // without holes, of 8^3-cell leaves each aligned to its own size, with ids
+    // of kBrickIdBits bits and value offsets of 31 bits.
+    const uint32_t* bricks;
     int32_t* err;           // the volume's Counters::error
 };
+
+constexpr int kBrickIdBits = 23;
+MB_HD uint32_t brick_word(int32_t leaf, int32_t shift) { return ((uint32_t)(127 - shift) << kBrickIdBits) | (uint32_t)leaf; }
 
 // Tetrahedral mesh as the kernels see it.  `g` carries the box
 // [0, hx) x [0, hy) x [0, hz) and every sampling and transfer-function

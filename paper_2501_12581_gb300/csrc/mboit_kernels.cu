@@ -297,6 +297,22 @@ __global__ void __launch_bounds__(256) k_check_ids(const int32_t* __restrict__ i
     flag_warp(bad, err, code);
 }
 
+// Every finest brick's leaf -1 or a leaf id, in the map and in the words
+// (whose other bits cannot lead an index astray).
+__global__ void __launch_bounds__(256) k_check_bricks(const int32_t* __restrict__ ids, const uint32_t* __restrict__ words,
+                                                      int64_t n, int32_t n_leaves, int32_t* err) {
+    bool bad = false;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i - threadIdx.x % 32 < n; i += stride) {
+        if (i < n) {
+            const int32_t v = __ldg(ids + i);
+            bad |= v < -1 || v >= n_leaves;
+            bad |= (int32_t)(__ldg(words + i) & ((1u << kBrickIdBits) - 1)) >= n_leaves;
+        }
+    }
+    flag_warp(bad, err, kErrLeafId);
+}
+
 // Every face neighbour -1 (boundary) or a tet id.
 __global__ void __launch_bounds__(256) k_check_nbrs(const int4* __restrict__ nb, int64_t n, int32_t n_tets,
                                                     int32_t* err) {
@@ -449,7 +465,10 @@ cudaError_t launch_sortlast_blend(const int64_t* base, int32_t* seg_key, float4*
 
 cudaError_t launch_check_tables(const AmrD& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.fdim * a.fdim * a.fdim;
-    k_check_ids<<<check_blocks(n), 256, 0, s>>>(a.fmap, n, -1, a.n_leaves - 1, a.err, kErrLeafId);
+    if (a.bricks)
+        k_check_bricks<<<check_blocks(n), 256, 0, s>>>(a.fmap, a.bricks, n, a.n_leaves, a.err);
+    else
+        k_check_ids<<<check_blocks(n), 256, 0, s>>>(a.fmap, n, -1, a.n_leaves - 1, a.err, kErrLeafId);
     return cudaGetLastError();
 }
 
