@@ -212,6 +212,54 @@ struct DepthRows {
     }
 };
 
+// Two consecutive lattice points (weight 1, the fixed step) added to the colour
+// C: table, opacity, weight T alpha and colour of both, each operation one
+// packed FP32x2 instruction with the scalar form's rounding, the colour sums
+// taken for a, then b, so that the result equals two one-point calls bit for
+// bit.  A point with ok = false adds nothing: its table coordinate is replaced
+// by 0 (no NaN enters) and its weight by 0, and fma(0, c, C) = C.  `live` false:
+// the pixel has no absorbance and its T may be NaN; nothing is added.  T():
+// both transmittances.
+template <class T>
+__device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float4& C, unsigned& n, float xa, float xb,
+                                           bool oka, bool okb, bool live, unsigned act, const T& transmittances) {
+    xa = oka ? xa : 0.0f;
+    xb = okb ? xb : 0.0f;
+    const int ia = (int)xa, ib = (int)xb;
+    const float fa = xa - (float)ia, fb = xb - (float)ib;
+    const float4 ea = s_tf[2 * ia], da = s_tf[2 * ia + 1], eb = s_tf[2 * ib], db = s_tf[2 * ib + 1];
+    // the table lerps as pairs: (r, g) and (b, absorbance) of each point
+    const float2 rga = __ffma2_rn(make_float2(fa, fa), make_float2(da.x, da.y), make_float2(ea.x, ea.y));
+    const float2 bwa = __ffma2_rn(make_float2(fa, fa), make_float2(da.z, da.w), make_float2(ea.z, ea.w));
+    const float2 rgb = __ffma2_rn(make_float2(fb, fb), make_float2(db.x, db.y), make_float2(eb.x, eb.y));
+    const float2 bwb = __ffma2_rn(make_float2(fb, fb), make_float2(db.z, db.w), make_float2(eb.z, eb.w));
+    const float2 a = make_float2(fmin_(bwa.y, amax), fmin_(bwb.y, amax));
+    // opacity 1 - e^-a: the series, and the direct form only when a lane of
+    // the branch has an absorbance at or above 1/4 (one_minus_exp_neg)
+    float2 p = __ffma2_rn(a, make_float2(-1.0f / 720.0f, -1.0f / 720.0f), make_float2(1.0f / 120.0f, 1.0f / 120.0f));
+    p = __ffma2_rn(a, p, make_float2(-1.0f / 24.0f, -1.0f / 24.0f));
+    p = __ffma2_rn(a, p, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
+    p = __ffma2_rn(a, p, make_float2(-0.5f, -0.5f));
+    p = __ffma2_rn(a, p, make_float2(1.0f, 1.0f));
+    float2 alpha = __fmul2_rn(a, p);
+    if (__any_sync(act, a.x >= 0.25f || a.y >= 0.25f)) {
+        const float2 ng = __fmul2_rn(a, make_float2(-kLog2e, -kLog2e));
+        const float2 dir = __ffma2_rn(make_float2(fexp2(ng.x), fexp2(ng.y)), make_float2(-1.0f, -1.0f),
+                                      make_float2(1.0f, 1.0f));
+        alpha = make_float2(a.x < 0.25f ? alpha.x : dir.x, a.y < 0.25f ? alpha.y : dir.y);
+    }
+    float2 wgt = __fmul2_rn(transmittances(), alpha);
+    wgt.x = oka && live ? wgt.x : 0.0f;
+    wgt.y = okb && live ? wgt.y : 0.0f;
+    // colour sums as pairs: (r, g) and (b, alpha); C.w + w = fma(w, 1, C.w)
+    float2 cxy = __ffma2_rn(make_float2(wgt.x, wgt.x), rga, make_float2(C.x, C.y));
+    float2 czw = __ffma2_rn(make_float2(wgt.x, wgt.x), make_float2(bwa.x, 1.0f), make_float2(C.z, C.w));
+    cxy = __ffma2_rn(make_float2(wgt.y, wgt.y), rgb, cxy);
+    czw = __ffma2_rn(make_float2(wgt.y, wgt.y), make_float2(bwb.x, 1.0f), czw);
+    C = make_float4(cxy.x, cxy.y, czw.x, czw.y);
+    n += (unsigned)oka + (unsigned)okb;
+}
+
 // Alg. 1 loop 2 per sample: colour += T(z) * alpha * (r, g, b, 1).
 struct BlendBody {
     const float4* s_tf;   // [2*i] = entry i (r, g, b, sigma*step), [2*i+1] = entry i+1 minus entry i
@@ -240,69 +288,38 @@ struct BlendBody {
     __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) { sample<false>(t, xt, ws); }
     __device__ __forceinline__ bool singular() const { return F.kind == kFrameOneAtom || F.kind == kFrameTwoAtoms; }
 
-    // Two consecutive lattice points (warped depths z.x, z.y; weight 1, the
-    // fixed step) of a generic frame: the arithmetic of sample<true> on both,
-    // each operation in one
-    // packed FP32x2 instruction with the scalar form's rounding, and the
-    // colour sums taken for a, then b.  The result equals two sample<true>
-    // calls bit for bit.  A point with ok = false adds nothing: its table
-    // coordinate is replaced by 0 (no NaN enters) and its weight by 0, and
-    // fma(0, c, C) = C.
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
-    __device__ __forceinline__ void pair_generic(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        xa = oka ? xa : 0.0f;
-        xb = okb ? xb : 0.0f;
-        const int ia = (int)xa, ib = (int)xb;
-        const float fa = xa - (float)ia, fb = xb - (float)ib;
-        const float4 ea = s_tf[2 * ia], da = s_tf[2 * ia + 1], eb = s_tf[2 * ib], db = s_tf[2 * ib + 1];
-        // the table lerps as pairs: (r, g) and (b, absorbance) of each point
-        const float2 rga = __ffma2_rn(make_float2(fa, fa), make_float2(da.x, da.y), make_float2(ea.x, ea.y));
-        const float2 bwa = __ffma2_rn(make_float2(fa, fa), make_float2(da.z, da.w), make_float2(ea.z, ea.w));
-        const float2 rgb = __ffma2_rn(make_float2(fb, fb), make_float2(db.x, db.y), make_float2(eb.x, eb.y));
-        const float2 bwb = __ffma2_rn(make_float2(fb, fb), make_float2(db.z, db.w), make_float2(eb.z, eb.w));
-        const float2 a = make_float2(fmin_(bwa.y, amax), fmin_(bwb.y, amax));
-        // opacity 1 - e^-a: the series, and the direct form only when a lane of
-        // the branch has an absorbance at or above 1/4 (one_minus_exp_neg)
-        float2 p = __ffma2_rn(a, make_float2(-1.0f / 720.0f, -1.0f / 720.0f), make_float2(1.0f / 120.0f, 1.0f / 120.0f));
-        p = __ffma2_rn(a, p, make_float2(-1.0f / 24.0f, -1.0f / 24.0f));
-        p = __ffma2_rn(a, p, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
-        p = __ffma2_rn(a, p, make_float2(-0.5f, -0.5f));
-        p = __ffma2_rn(a, p, make_float2(1.0f, 1.0f));
-        float2 alpha = __fmul2_rn(a, p);
-        if (__any_sync(act, a.x >= 0.25f || a.y >= 0.25f)) {
-            const float2 ng = __fmul2_rn(a, make_float2(-kLog2e, -kLog2e));
-            const float2 dir = __ffma2_rn(make_float2(fexp2(ng.x), fexp2(ng.y)), make_float2(-1.0f, -1.0f),
-                                          make_float2(1.0f, 1.0f));
-            alpha = make_float2(a.x < 0.25f ? alpha.x : dir.x, a.y < 0.25f ? alpha.y : dir.y);
-        }
-        const float2 A = bound_generic2(F, z, w0, act);
-        const float2 ex = __fmul2_rn(make_float2(-F.m0_log2e, -F.m0_log2e), A);
-        float2 wgt = __fmul2_rn(make_float2(fexp2(ex.x), fexp2(ex.y)), alpha);
-        wgt.x = oka ? wgt.x : 0.0f;
-        wgt.y = okb ? wgt.y : 0.0f;
-        // colour sums as pairs: (r, g) and (b, alpha); C.w + w = fma(w, 1, C.w)
-        float2 cxy = __ffma2_rn(make_float2(wgt.x, wgt.x), rga, make_float2(C.x, C.y));
-        float2 czw = __ffma2_rn(make_float2(wgt.x, wgt.x), make_float2(bwa.x, 1.0f), make_float2(C.z, C.w));
-        cxy = __ffma2_rn(make_float2(wgt.y, wgt.y), rgb, cxy);
-        czw = __ffma2_rn(make_float2(wgt.y, wgt.y), make_float2(bwb.x, 1.0f), czw);
-        C = make_float4(cxy.x, cxy.y, czw.x, czw.y);
-        n += (unsigned)oka + (unsigned)okb;
+    // Frames whose points pair_generic may take: generic ones, and pixels
+    // without absorbance, whose opacities are all 0 (T is finite there).
+    __device__ __forceinline__ bool pairs() const { return F.kind == kFrameGeneric || F.kind == kFrameEmpty; }
+    // Two points of a generic frame: equal to two sample<true> calls bit for bit.
+    __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, true, act, [&]() {
+            const float2 ex = __fmul2_rn(make_float2(-F.m0_log2e, -F.m0_log2e), bound_generic2(F, z, w0, act));
+            return make_float2(fexp2(ex.x), fexp2(ex.y));
+        });
     }
 };
 
-// The pass-2 body for a warp whose lanes with samples all have a generic
-// frame: the same operations without the per-sample test of the frame's kind.
-struct GenericBlend {
-    BlendBody& b;
-    __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) { b.sample<true>(t, xt, ws); }
+// A pass-2 body in a warp whose lanes with samples all may take two points at
+// once (pairs()).
+template <class Body>
+struct PairBlend {
+    Body& b;
+    __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) {
+        if constexpr (std::is_same<Body, BlendBody>::value)
+            b.template sample<true>(t, xt, ws);   // no test of the frame's kind
+        else
+            b(t, xt, ws);
+    }
     __device__ __forceinline__ float depth(float t) const { return b.depth(t); }
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        b.pair_generic(z, xa, xb, oka, okb, act);
+        b.pair(z, xa, xb, oka, okb, act);
     }
 };
 // Bodies that take two lattice points at once (pair(...), equal to two calls).
 template <class B> struct HasPair : std::false_type {};
-template <> struct HasPair<GenericBlend> : std::true_type {};
+template <class B> struct HasPair<PairBlend<B>> : std::true_type {};
 // Bodies that are told the unit (brick or tet) of every point before its
 // sample, and may decline it (bool enter(int unit)).
 template <class B> struct TakesUnits : std::false_type {};
@@ -311,8 +328,9 @@ template <class B> struct TakesUnits : std::false_type {};
 // power moments and of trigonometric moments (root solves, series) take the
 // loop rolled: 8 or 16 inlined copies of them overflow the instruction cache
 // (octree frame with 8 power moments: 103 ms unrolled by 8, 219 ms by 16).
-template <class B> struct RowUnroll : std::integral_constant<bool, HasPair<B>::value> {};
+template <class B> struct RowUnroll : std::false_type {};
 template <> struct RowUnroll<BlendBody> : std::true_type {};
+template <class B> struct RowUnroll<PairBlend<B>> : RowUnroll<B> {};
 
 // Bytes of one moment slab of P pixels in the volume's format.
 __device__ __forceinline__ int64_t slab_bytes(const GridD& g, int plane) {
@@ -388,6 +406,12 @@ struct TrigMomentBody {
     }
 };
 
+// T = e^(-b0 A) of two points, clamped to [0, 1] as the one-point bodies do.
+__device__ __forceinline__ float2 heavy_transmittance(float m0_log2e, float2 A) {
+    const float2 ex = __fmul2_rn(make_float2(-m0_log2e, -m0_log2e), A);
+    return make_float2(fclamp(fexp2(ex.x), 0.0f, 1.0f), fclamp(fexp2(ex.y), 0.0f, 1.0f));
+}
+
 // Pass 2 with trigonometric moments.
 template <int N>
 struct TrigBlendBody {
@@ -405,7 +429,7 @@ struct TrigBlendBody {
         const float a = fmin_(ffma(f, de.w, e0.w) * ws, amax);
         const float alpha = one_minus_exp_neg(a);
         const float z = warp_depth(t, wa, wb);
-        const float A = trig_fraction<N>(F, *T, z, w0);
+        const float A = F.n == 0 ? 0.0f : trig_fraction<N, float>(F, *T, z, w0);
         const float wgt = fclamp(fexp2(-F.m0_log2e * A), 0.0f, 1.0f) * alpha;
         C.x = ffma(wgt, ffma(f, de.x, e0.x), C.x);
         C.y = ffma(wgt, ffma(f, de.y, e0.y), C.y);
@@ -414,6 +438,12 @@ struct TrigBlendBody {
         ++n;
     }
     __device__ __forceinline__ bool singular() const { return b0 > 0.0f && F.n == 0; }
+    __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
+    __device__ __forceinline__ bool pairs() const { return !singular(); }
+    __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.n != 0, act,
+                   [&]() { return heavy_transmittance(F.m0_log2e, trig_fraction<N, float2>(F, *T, z, w0)); });
+    }
 };
 
 // Slab of 2N power moments: b0 plane (float), the float4 plane of b1..b4,
@@ -496,6 +526,12 @@ struct PowerBlendBody {
         ++n;
     }
     __device__ __forceinline__ bool singular() const { return F.kind == kFrameFourMoments; }
+    __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
+    __device__ __forceinline__ bool pairs() const { return !singular(); }
+    __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.kind == kFrameGeneric, act,
+                   [&]() { return heavy_transmittance(F.m0_log2e, power_fraction_generic<N, float2>(F, z, w0)); });
+    }
 };
 
 template <int MS> struct Bodies;
@@ -727,25 +763,41 @@ __device__ __forceinline__ void march_rows(const GridD& g, const float* __restri
         __syncwarp();
         const float* src = buf + (c & 1) * kRowChunk * 32 + lane;
         const int n = min(kRowChunk, kmax - kc + 1);
-        if (kc >= k0 && kc + kRowChunk - 1 <= k1) {
+        if constexpr (HasPair<Body>::value && !kTagged) {
+            // two lattice points per call (packed FP32x2 arithmetic).  (The
+            // adaptive step leaves most points unsampled, lane-coherently: there
+            // the single-point loop below skips more.)
+            const float2* zr = reinterpret_cast<const float2*>(buf + kRowZ);
+            const bool any = k0 <= k1, whole = kc >= k0 && kc + kRowChunk - 1 <= k1;
+            if (__all_sync(0xffffffffu, whole || !any)) {
+                // the whole chunk lies in every lane's interval (and, without a
+                // selection, every point of it is owned)
+                if (any) {
+                    const unsigned act = __activemask();
+#pragma unroll(RowUnroll<Body>::value ? kRowChunk / 2 : 1)
+                    for (int i = 0; i < kRowChunk; i += 2) {
+                        const float va = src[i * 32], vb = src[(i + 1) * 32];
+                        const bool oka = !kSel || va == va, okb = !kSel || vb == vb;
+                        if (kSel && !__any_sync(act, oka || okb)) continue;   // a pair no lane samples
+                        body.pair(zr[i / 2], va, vb, oka, okb, act);
+                    }
+                }
+            } else {
+                // the ends of the rays: points outside a lane's interval add nothing
+#pragma unroll 1
+                for (int i = 0; i < n; i += 2) {
+                    const int k = kc + i;
+                    const float va = src[i * 32], vb = src[(i + 1) * 32];
+                    const bool oka = k >= k0 && k <= k1 && (!kSel || va == va);
+                    const bool okb = k + 1 >= k0 && k + 1 <= k1 && (!kSel || vb == vb);
+                    if (!__any_sync(0xffffffffu, oka || okb)) continue;
+                    body.pair(zr[i / 2], va, vb, oka, okb, 0xffffffffu);
+                }
+            }
+        } else if (kc >= k0 && kc + kRowChunk - 1 <= k1) {
             // the whole chunk lies in this lane's interval (and, without a
             // selection, every point of it is owned)
-            if constexpr (HasPair<Body>::value && !kTagged) {
-                // two lattice points per call (packed FP32x2 arithmetic); with a
-                // selection, a pair no lane of this branch samples is skipped.
-                // (The adaptive step leaves most points unsampled, lane-coherently:
-                // there the single-point loop below skips more.)
-                const unsigned act = __activemask();
-                const float2* zr = reinterpret_cast<const float2*>(buf + kRowZ);
-#pragma unroll
-                for (int i = 0; i < kRowChunk; i += 2) {
-                    const float va = src[i * 32], vb = src[(i + 1) * 32];
-                    const bool oka = !kSel || va == va, okb = !kSel || vb == vb;
-                    if (kSel && !__any_sync(act, oka || okb)) continue;
-                    body.pair(zr[i / 2], va, vb, oka, okb, act);
-                }
-                t += kRowChunk * g.step;
-            } else if constexpr (RowUnroll<Body>::value) {
+            if constexpr (RowUnroll<Body>::value) {
 #pragma unroll
                 for (int i = 0; i < kRowChunk; ++i, t += g.step) {
                     const float val = src[i * 32];
@@ -778,19 +830,15 @@ __device__ __forceinline__ void march_rows(const GridD& g, const float* __restri
     }
 }
 
-// Pass 2 from the tile's cache rows.  With four power moments, a warp whose
-// lanes with samples all have a generic frame (lanes without samples never
-// call the body) takes the loop without the per-sample test of the frame's
-// kind; the arithmetic, and so the result, is the same.
+// Pass 2 from the tile's cache rows, two points at a time in a warp whose lanes
+// with samples all may (pairs(); lanes without samples never call the body).
 template <bool kSel, bool kTagged = false, int kChunk = kRowChunk, class Body>
 __device__ __forceinline__ void blend_rows(const GridD& g, const float* __restrict__ rows, int kmin, int kmax, int k0,
                                            int k1, float* __restrict__ buf, Body& body, int tmask = 0) {
-    if constexpr (std::is_same<Body, BlendBody>::value) {
-        if (__all_sync(0xffffffffu, k0 > k1 || body.F.kind == kFrameGeneric)) {
-            GenericBlend gb{body};
-            march_rows<kSel, GenericBlend, kTagged, kChunk>(g, rows, kmin, kmax, k0, k1, buf, gb, tmask);
-            return;
-        }
+    if (__all_sync(0xffffffffu, k0 > k1 || body.pairs())) {
+        PairBlend<Body> pb{body};
+        march_rows<kSel, PairBlend<Body>, kTagged, kChunk>(g, rows, kmin, kmax, k0, k1, buf, pb, tmask);
+        return;
     }
     march_rows<kSel, Body, kTagged, kChunk>(g, rows, kmin, kmax, k0, k1, buf, body, tmask);
 }

@@ -328,7 +328,7 @@ __device__ __forceinline__ bool blend_fused(const GridD& g, const uint8_t* __res
                                             TmaWin* tma = nullptr) {
     if constexpr (std::is_same<Body, BlendBody>::value) {
         if (__all_sync(0xffffffffu, k0 > k1 || body.F.kind == kFrameGeneric)) {
-            GenericBlend gb{body};
+            PairBlend<BlendBody> gb{body};
             return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, gb, NoStore{}, tma);
         }
     }

@@ -14,9 +14,10 @@
 //   per sample, FP32: y = L^-1 v(x0), K(x0, x0) = sum y_k^2 / D_k,
 //     q = L^-T D^-1 y (the kernel polynomial K(., x0) = sum q_j x^j), its n
 //     real roots in the variable s = 1 / (x - x0) from closed forms (Viete,
-//     Ferrari) polished by Newton steps, and the Christoffel weight
-//     1 / K(x_i, x_i) of every root in front:
-//     A = w0 / K(x0, x0) + sum_{x_i < x0} 1 / K(x_i, x_i).
+//     Ferrari) polished by Newton steps, and the Christoffel weights
+//     1 / K(x_i, x_i) of the roots in front,
+//     A = w0 / K(x0, x0) + sum_{x_i < x0} 1 / K(x_i, x_i),
+//     or, where fewer roots lie behind, 1 less their weights (front_weight).
 // Every weight is a sum of positive terms, so no cancellation enters A.  A
 // pixel whose Hankel matrix is numerically singular (a pivot below 1e-12 of
 // its diagonal entry: no bias and at most n absorbers) falls back to the
@@ -119,44 +120,53 @@ MB_HD PowerFrame<N> make_power_frame(const float* m_in, float moment_bias) {
 }
 
 // K(x, x) = sum_k (L^-1 v(x))_k^2 / D_k.
-template <int N>
-MB_HD float power_kernel_diag(const PowerFrame<N>& P, float x) {
-    float y[N + 1], v = 1.0f, K = 0.0f;
+template <int N, class T>
+MB_HD T power_kernel_diag(const PowerFrame<N>& P, T x) {
+    T y[N + 1], v = Vec<T>::splat(1.0f), K = Vec<T>::splat(0.0f);
 #pragma unroll
     for (int i = 0; i <= N; ++i) {
-        float t = v;
+        T t = v;
 #pragma unroll
-        for (int k = 0; k < i; ++k) t = ffma(-P.L[i * (i - 1) / 2 + k], y[k], t);
+        for (int k = 0; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), y[k], t);
         y[i] = t;
-        K = ffma(t * t, P.invD[i], K);
-        v *= x;
+        K = vfma(vmul(t, t), Vec<T>::splat(P.invD[i]), K);
+        v = vmul(v, x);
     }
     return K;
 }
 
-// Alg. 3 at order N: fraction A of the optical depth in front of warped
-// depth z0.
-template <int N>
-MB_HD float power_fraction(const PowerFrame<N>& P, float z0, float w0) {
-    if (P.kind != kFrameGeneric) return P.kind == kFrameEmpty ? 0.0f : bound_fraction(P.F4, z0, w0);
-    const float x0 = ffma(z0, P.inv_s, P.nmu);
-    float u[N + 1], y[N + 1], v = 1.0f, K00 = 0.0f;
+// Weight of the support point at x0 + 1/s.  A point with |s| < 1e-4 lies beyond
+// |x - x0| = 1e4: its weight, below 1e-30, is not worth an overflow.
+template <int N, class T>
+MB_HD T power_weight(const PowerFrame<N>& P, T x0, T s) {
+    const T lim = Vec<T>::splat(1e-4f);
+    const Lanes<T> far = below(s, lim) + below(vneg(s), lim);    // 2: both
+    const T w = vrcp(power_kernel_diag<N, T>(P, vadd(x0, vrcp(s))));
+    return pick_eq(far, 2, Vec<T>::splat(0.0f), w);
+}
+
+// Alg. 3 at order N for a generic frame: fraction A of the optical depth in
+// front of warped depth z0, for one depth (float) or two (float2).
+template <int N, class T>
+MB_HD T power_fraction_generic(const PowerFrame<N>& P, T z0, float w0) {
+    const T x0 = vfma(z0, Vec<T>::splat(P.inv_s), Vec<T>::splat(P.nmu));
+    T u[N + 1], y[N + 1], v = Vec<T>::splat(1.0f), K00 = Vec<T>::splat(0.0f);
 #pragma unroll
     for (int i = 0; i <= N; ++i) {
-        float t = v;
+        T t = v;
 #pragma unroll
-        for (int k = 0; k < i; ++k) t = ffma(-P.L[i * (i - 1) / 2 + k], u[k], t);
+        for (int k = 0; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), u[k], t);
         u[i] = t;
-        y[i] = t * P.invD[i];
-        K00 = ffma(t, y[i], K00);
-        v *= x0;
+        y[i] = vmul(t, Vec<T>::splat(P.invD[i]));
+        K00 = vfma(t, y[i], K00);
+        v = vmul(v, x0);
     }
     // q = L^-T D^-1 y: coefficients of K(., x0) in the standardised frame
 #pragma unroll
     for (int i = N - 1; i >= 0; --i) {
-        float t = y[i];
+        T t = y[i];
 #pragma unroll
-        for (int k = i + 1; k <= N; ++k) t = ffma(-P.L[k * (k - 1) / 2 + i], y[k], t);
+        for (int k = i + 1; k <= N; ++k) t = vfma(Vec<T>::splat(-P.L[k * (k - 1) / 2 + i]), y[k], t);
         y[i] = t;
     }
     // Substituting x = x0 + 1/s sends x0 to s = infinity: s^N K(x0 + 1/s, x0)
@@ -168,21 +178,25 @@ MB_HD float power_fraction(const PowerFrame<N>& P, float z0, float w0) {
 #pragma unroll
     for (int k = 0; k < N; ++k)
 #pragma unroll
-        for (int i = N - 1; i >= k; --i) y[i] = ffma(x0, y[i + 1], y[i]);
-    const float iK = frcp(K00);
-    float rts[N];
-    if (N == 3)
-        cubic3(y[1] * iK, y[2] * iK, y[3] * iK, rts);
+        for (int i = N - 1; i >= k; --i) y[i] = vfma(x0, y[i + 1], y[i]);
+    const T rho0 = vrcp(K00);
+    T rts[N];
+    if constexpr (N == 3)
+        cubic3(vmul(y[1], rho0), vmul(y[2], rho0), vmul(y[3], rho0), rts);
     else
-        quartic4(y[1] * iK, y[2] * iK, y[3] * iK, y[4] * iK, rts);
-    float A = w0 * iK;
+        quartic4(vmul(y[1], rho0), vmul(y[2], rho0), vmul(y[3], rho0), vmul(y[4], rho0), rts);
+    const T zero = Vec<T>::splat(0.0f), one = Vec<T>::splat(1.0f);
+    Lanes<T> front = below(rts[0], zero);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-        // |s| < 1e-4: a point beyond |x - x0| = 1e4, weight below 1e-30
-        if (!(rts[i] < -1e-4f)) continue;
-        A += frcp(power_kernel_diag<N>(P, x0 + frcp(rts[i])));
-    }
-    return fclamp(A, 0.0f, 1.0f);
+    for (int i = 1; i < N; ++i) front = front + below(rts[i], zero);
+    const T A = front_weight<N, T>(rts, front, rho0, Vec<T>::splat(w0), [&](T s) { return power_weight<N, T>(P, x0, s); });
+    return vmin(vmax(A, zero), one);
+}
+
+template <int N>
+MB_HD float power_fraction(const PowerFrame<N>& P, float z0, float w0) {
+    if (P.kind != kFrameGeneric) return P.kind == kFrameEmpty ? 0.0f : bound_fraction(P.F4, z0, w0);
+    return power_fraction_generic<N, float>(P, z0, w0);
 }
 
 }  // namespace mb

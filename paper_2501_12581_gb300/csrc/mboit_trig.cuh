@@ -23,29 +23,40 @@
 // arithmetic is FP32.  The conditioning of G is bounded by the bias (about
 // 1 / beta); the 16-bit storages need beta >= 2e-3, where FP32 suffices.
 #pragma once
-#include "mboit_device.cuh"
+#include "mboit_vec.cuh"
 
 namespace mb {
-
-MB_HD float fcos(float x) {
-#if defined(__CUDA_ARCH__)
-    return __cosf(x);
-#else
-    return cosf(x);
-#endif
-}
 
 struct cf {
     float x, y;
 };
 MB_HD cf cmul(cf a, cf b) { return {ffma(a.x, b.x, -a.y * b.y), ffma(a.x, b.y, a.y * b.x)}; }
 MB_HD cf cconj(cf a) { return {a.x, -a.y}; }
-MB_HD cf csub(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
-MB_HD cf cscale(cf a, float s) { return {a.x * s, a.y * s}; }
+
+// Complex numbers of one point or two (mboit_vec.cuh), by coefficients that the
+// points of a pixel share.
+template <class T>
+struct cv {
+    T x, y;
+};
+template <class T>
+MB_HD cv<T> cmul(cv<T> a, cv<T> b) {
+    return {vfma(a.x, b.x, vmul(vneg(a.y), b.y)), vfma(a.x, b.y, vmul(a.y, b.x))};
+}
+template <class T>
+MB_HD cv<T> cconj(cv<T> a) { return {a.x, vneg(a.y)}; }
 // a - b * c
-MB_HD cf cfms(cf a, cf b, cf c) { return {ffma(-b.x, c.x, ffma(b.y, c.y, a.x)), ffma(-b.x, c.y, ffma(-b.y, c.x, a.y))}; }
+template <class T>
+MB_HD cv<T> cfms(cv<T> a, cf b, cv<T> c) {
+    const T nx = Vec<T>::splat(-b.x), y = Vec<T>::splat(b.y), ny = Vec<T>::splat(-b.y);
+    return {vfma(nx, c.x, vfma(y, c.y, a.x)), vfma(nx, c.y, vfma(ny, c.x, a.y))};
+}
 // a - conj(b) * c
-MB_HD cf cfms_conj(cf a, cf b, cf c) { return {ffma(-b.x, c.x, ffma(-b.y, c.y, a.x)), ffma(-b.x, c.y, ffma(b.y, c.x, a.y))}; }
+template <class T>
+MB_HD cv<T> cfms_conj(cv<T> a, cf b, cv<T> c) {
+    const T nx = Vec<T>::splat(-b.x), y = Vec<T>::splat(b.y), ny = Vec<T>::splat(-b.y);
+    return {vfma(nx, c.x, vfma(ny, c.y, a.x)), vfma(nx, c.y, vfma(y, c.x, a.y))};
+}
 
 struct TrigFrame {
     int32_t n;            // 0: no absorber, or G not positive definite (then A = 0)
@@ -99,168 +110,127 @@ MB_HD TrigFrame make_trig_frame(float b0, const cf* tau, int n, float beta) {
     return F;
 }
 
-// Real roots of the monic cubic s^3 + a s^2 + b s + c whose roots are all
-// real (Viete's trigonometric form), then one Newton step each.
-MB_HD void cubic3(float a, float b, float c, float r[3]) {
-    const float a3 = a * (1.0f / 3.0f);
-    const float p = ffma(-a, a3, b);
-    const float q = ffma(ffma(2.0f * a3, a3, -b), a3, c);  // 2 a3^3 - b a3 + c
-    const float pm = fmin_(p, -1e-30f);
-    const float m = 2.0f * fsqrt_fast(-pm * (1.0f / 3.0f));
-    const float arg = fclamp(fdiv_fast(3.0f * q, pm * m), -1.0f, 1.0f);
-    const float th = acosf(arg) * (1.0f / 3.0f);  // th in [0, pi/3]: the fast cosine is accurate on this range
-    const float k2 = 2.0943951023931957f;  // 2 pi / 3
-    r[0] = ffma(m, fcos(th), -a3);
-    r[1] = ffma(m, fcos(th - k2), -a3);
-    r[2] = ffma(m, fcos(th + k2), -a3);
-    for (int i = 0; i < 3; ++i) {
-        const float s = r[i];
-        const float f = ffma(ffma(s + a, s, b), s, c);
-        const float df = ffma(ffma(3.0f, s, 2.0f * a), s, b);
-        if (df != 0.0f) r[i] = s - fdiv_fast(f, df);   // Newton corrects the 2-ulp quotient
-    }
+MB_HD void sincos_fast(float x, float& sn, float& cs) {
+#if defined(__CUDA_ARCH__)
+    __sincosf(x, &sn, &cs);
+#else
+    sn = sinf(x);
+    cs = cosf(x);
+#endif
 }
-
-// The largest real root of the monic cubic s^3 + a s^2 + b s + c whose roots
-// are all real: Viete's root of the largest cosine (th in [0, pi/3]), then one
-// Newton step.
-MB_HD float cubic3_max(float a, float b, float c) {
-    const float a3 = a * (1.0f / 3.0f);
-    const float p = ffma(-a, a3, b);
-    const float q = ffma(ffma(2.0f * a3, a3, -b), a3, c);
-    const float pm = fmin_(p, -1e-30f);
-    const float m = 2.0f * fsqrt_fast(-pm * (1.0f / 3.0f));
-    const float arg = fclamp(fdiv_fast(3.0f * q, pm * m), -1.0f, 1.0f);
-    const float s = ffma(m, fcos(acosf(arg) * (1.0f / 3.0f)), -a3);
-    const float f = ffma(ffma(s + a, s, b), s, c);
-    const float df = ffma(ffma(3.0f, s, 2.0f * a), s, b);
-    return df != 0.0f ? s - fdiv_fast(f, df) : s;
+#if defined(__CUDACC__)
+__device__ __forceinline__ void sincos_fast(float2 x, float2& sn, float2& cs) {
+    sincos_fast(x.x, sn.x, cs.x);
+    sincos_fast(x.y, sn.y, cs.y);
 }
-
-// Real roots of the monic quartic s^4 + a s^3 + b s^2 + c s + d whose roots
-// are all real (Ferrari: resolvent cubic, two quadratics), then Newton steps.
-MB_HD void quartic4(float a, float b, float c, float d, float r[4]) {
-    const float a4 = 0.25f * a;
-    const float a42 = a4 * a4;
-    const float p = ffma(-6.0f, a42, b);
-    const float q = ffma(ffma(8.0f, a42, -2.0f * b), a4, c);              // c - 2 b a4 + 8 a4^3
-    const float rr = ffma(ffma(ffma(-3.0f, a42, b), a4, -c), a4, d);      // d - c a4 + b a4^2 - 3 a4^4
-    float y[4];
-    const float scale = fmax_(fabsf(p), fmax_(fsqrt_fast(fabsf(rr)), 1e-30f));
-    if (fabsf(q) <= 1e-6f * scale * fsqrt_fast(scale)) {
-        // biquadratic: y^2 = (-p +- sqrt(p^2 - 4 r)) / 2
-        const float disc = fsqrt_fast(fmax_(ffma(p, p, -4.0f * rr), 0.0f));
-        const float y1 = fsqrt_fast(fmax_(0.5f * (-p + disc), 0.0f));
-        const float y2 = fsqrt_fast(fmax_(0.5f * (-p - disc), 0.0f));
-        y[0] = -y1; y[1] = -y2; y[2] = y2; y[3] = y1;
-    } else {
-        // m^3 + p m^2 + (p^2/4 - r) m - q^2/8 = 0, largest root (positive)
-        const float m = fmax_(cubic3_max(p, ffma(0.25f * p, p, -rr), -0.125f * q * q), 1e-30f);
-        const float sq = fsqrt_fast(2.0f * m);
-        const float h = 0.5f * p + m, g = fdiv_fast(q, 2.0f * sq);
-        // y^2 - sq y + (h + g) = 0 and y^2 + sq y + (h - g) = 0
-        const float d1 = fsqrt_fast(fmax_(ffma(sq, sq, -4.0f * (h + g)), 0.0f));
-        const float d2 = fsqrt_fast(fmax_(ffma(sq, sq, -4.0f * (h - g)), 0.0f));
-        y[0] = 0.5f * (sq - d1); y[1] = 0.5f * (sq + d1);
-        y[2] = 0.5f * (-sq - d2); y[3] = 0.5f * (-sq + d2);
-    }
-    for (int i = 0; i < 4; ++i) {
-        float s = y[i] - a4;
-        for (int it = 0; it < 1; ++it) {
-            const float f = ffma(ffma(ffma(s + a, s, b), s, c), s, d);
-            const float df = ffma(ffma(ffma(4.0f, s, 3.0f * a), s, 2.0f * b), s, c);
-            if (df != 0.0f) s = s - fdiv_fast(f, df);
-        }
-        r[i] = s;
-    }
-}
+#endif
 
 // K(u, u) = sum_k |x_k|^2 / D_k with L x = conj(v(u)).
-template <int N>
-MB_HD float trig_kernel_diag(const TrigFrame& F, cf u) {
-    cf x[N + 1];
-    cf ub = cconj(u), p = {1.0f, 0.0f};
-    float K = 0.0f;
+template <int N, class T>
+MB_HD T trig_kernel_diag(const TrigFrame& F, cv<T> u) {
+    cv<T> x[N + 1];
+    cv<T> ub = cconj(u), p = {Vec<T>::splat(1.0f), Vec<T>::splat(0.0f)};
+    T K = Vec<T>::splat(0.0f);
 #pragma unroll
     for (int i = 0; i <= N; ++i) {
-        cf xi = p;
+        cv<T> xi = p;
 #pragma unroll
         for (int k = 0; k < i; ++k) xi = cfms(xi, F.L[i * (i - 1) / 2 + k], x[k]);
         x[i] = xi;
-        K = ffma(ffma(xi.x, xi.x, xi.y * xi.y), F.invD[i], K);
+        K = vfma(vfma(xi.x, xi.x, vmul(xi.y, xi.y)), Vec<T>::splat(F.invD[i]), K);
         p = cmul(p, ub);
     }
     return K;
 }
 
+// Weight of the node at s: 1 / K(u, u) at u = u0 (s + i) / (s - i).
+template <int N, class T>
+MB_HD T trig_weight(const TrigFrame& F, cv<T> u0, T s) {
+    const T one = Vec<T>::splat(1.0f);
+    const T s2 = vmul(s, s);
+    const T inv = vrcp(vadd(s2, one));
+    const cv<T> e = {vmul(vsub(s2, one), inv), vmul(vadd(s, s), inv)};
+    return vrcp(trig_kernel_diag<N, T>(F, cmul(u0, e)));
+}
+
+// Sum of the weights of the nodes in front, r ascending, the first `front` of
+// them in front; `weight` gives a root's.  The weights of all nodes and of the
+// point itself (rho0) add up to 1, so the smaller side is summed: one weight
+// of three nodes, at most two of four (the second only where a point of the
+// warp has two nodes on either side), instead of every one in front.
+template <int N, class T, class W>
+MB_HD T front_weight(const T* r, Lanes<T> front, T rho0, T w0, const W& weight) {
+    const T one = Vec<T>::splat(1.0f), zero = Vec<T>::splat(0.0f);
+    const T lo = vmul(w0, rho0), hi = vfma(vsub(w0, one), rho0, one);
+    // the side's outermost node, none where the other side holds all
+    const T s = pick_gt(front, N / 2, r[N - 1], r[0]);
+    T w = weight(s);
+    w = pick_eq(front, 0, zero, pick_eq(front, N, zero, w));
+    if (N == 4 && any_eq(front, 2)) w = vadd(w, pick_eq(front, 2, weight(r[1]), zero));
+    return pick_gt(front, N / 2, vsub(hi, w), vadd(lo, w));
+}
+
 // Alg. 3 for trigonometric moments: fraction A of the optical depth in front
-// of warped depth z0.
-template <int N>
-MB_HD float trig_fraction(const TrigFrame& F, const TrigTables& T, float z0, float w0) {
-    if (F.n == 0) return 0.0f;
-    const float phi = z0 * T.zone_scale;
-#if defined(__CUDA_ARCH__)
-    float sn, cs;
-    __sincosf(phi, &sn, &cs);
-#else
-    const float sn = sinf(phi), cs = cosf(phi);
-#endif
-    const cf u0 = {cs, sn};
+// of warped depth z0 (F.n > 0), for one depth (float) or two (float2).
+template <int N, class T>
+MB_HD T trig_fraction(const TrigFrame& F, const TrigTables& tab, T z0, float w0) {
+    cv<T> u0;
+    sincos_fast(vmul(z0, Vec<T>::splat(tab.zone_scale)), u0.y, u0.x);
     // y = G^-1 w, w = conj(v(u0)) = (1, conj(u0), conj(u0)^2, ..)
-    cf w[N + 1], y[N + 1];
-    w[0] = {1.0f, 0.0f};
+    cv<T> w[N + 1], y[N + 1];
+    w[0] = {Vec<T>::splat(1.0f), Vec<T>::splat(0.0f)};
+    w[1] = cconj(u0);
 #pragma unroll
-    for (int k = 1; k <= N; ++k) w[k] = cmul(w[k - 1], cconj(u0));
+    for (int k = 2; k <= N; ++k) w[k] = cmul(w[k - 1], w[1]);
 #pragma unroll
     for (int i = 0; i <= N; ++i) {
-        cf t = w[i];
+        cv<T> t = w[i];
 #pragma unroll
         for (int k = 0; k < i; ++k) t = cfms(t, F.L[i * (i - 1) / 2 + k], y[k]);
         y[i] = t;
     }
 #pragma unroll
-    for (int i = 0; i <= N; ++i) y[i] = cscale(y[i], F.invD[i]);
+    for (int i = 0; i <= N; ++i) {
+        const T d = Vec<T>::splat(F.invD[i]);
+        y[i] = {vmul(y[i].x, d), vmul(y[i].y, d)};
+    }
 #pragma unroll
     for (int i = N; i >= 0; --i) {
-        cf t = y[i];
+        cv<T> t = y[i];
 #pragma unroll
         for (int k = i + 1; k <= N; ++k) t = cfms_conj(t, F.L[k * (k - 1) / 2 + i], y[k]);
         y[i] = t;
     }
     // z_k = y_k u0^k; K(u0, u0) = Re sum z_k; real polynomial coefficients
-    float zr[N + 1], zi[N + 1], K00 = 0.0f;
+    T zr[N + 1], nzi[N + 1], K00 = Vec<T>::splat(0.0f);
 #pragma unroll
     for (int k = 0; k <= N; ++k) {
-        const cf z = cmul(y[k], cconj(w[k]));
+        const cv<T> z = cmul(y[k], cconj(w[k]));
         zr[k] = z.x;
-        zi[k] = z.y;
-        K00 += z.x;
+        nzi[k] = vneg(z.y);
+        K00 = vadd(K00, z.x);
     }
-    const float invK = frcp(K00);
-    float coef[N];
+    const T rho0 = vrcp(K00);
+    T coef[N];
 #pragma unroll
     for (int m = 0; m < N; ++m) {
-        float acc = 0.0f;
+        T acc = Vec<T>::splat(0.0f);
 #pragma unroll
-        for (int k = 0; k <= N; ++k) acc = ffma(zr[k], T.er[k][m], ffma(-zi[k], T.ei[k][m], acc));
-        coef[m] = acc * invK;
+        for (int k = 0; k <= N; ++k)
+            acc = vfma(zr[k], Vec<T>::splat(tab.er[k][m]), vfma(nzi[k], Vec<T>::splat(tab.ei[k][m]), acc));
+        coef[m] = vmul(acc, rho0);
     }
-    float rts[N];
-    if (N == 3)
+    T rts[N];
+    if constexpr (N == 3)
         cubic3(coef[2], coef[1], coef[0], rts);
     else
         quartic4(coef[3], coef[2], coef[1], coef[0], rts);
-    const float sp = sn / (1.0f + cs);  // tan(phi0 / 2); |phi0| < pi by the wrapping zone
-    float A = w0 * invK;
+    // tan(phi0 / 2); |phi0| < pi by the wrapping zone
+    const T sp = vmul(u0.y, vrcp(vadd(Vec<T>::splat(1.0f), u0.x)));
+    Lanes<T> front = below(rts[0], sp);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const float s = rts[i];
-        if (!(s < sp)) continue;
-        const float inv = frcp(ffma(s, s, 1.0f));
-        const cf e = {(s * s - 1.0f) * inv, 2.0f * s * inv};  // (s + i) / (s - i)
-        A += frcp(trig_kernel_diag<N>(F, cmul(u0, e)));
-    }
-    return A;
+    for (int i = 1; i < N; ++i) front = front + below(rts[i], sp);
+    return front_weight<N, T>(rts, front, rho0, Vec<T>::splat(w0), [&](T s) { return trig_weight<N, T>(F, u0, s); });
 }
 
 }  // namespace mb
