@@ -282,7 +282,7 @@ struct BlendBody {
         C.x = ffma(wgt, ffma(f, de.x, e0.x), C.x);
         C.y = ffma(wgt, ffma(f, de.y, e0.y), C.y);
         C.z = ffma(wgt, ffma(f, de.z, e0.z), C.z);
-        C.w += wgt;
+        C.w = fadd(C.w, wgt);   // not contracted with the product: as in blend_pair
         ++n;
     }
     __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) { sample<false>(t, xt, ws); }
@@ -430,11 +430,11 @@ struct TrigBlendBody {
         const float alpha = one_minus_exp_neg(a);
         const float z = warp_depth(t, wa, wb);
         const float A = F.n == 0 ? 0.0f : trig_fraction<N, float>(F, *T, z, w0);
-        const float wgt = fclamp(fexp2(-F.m0_log2e * A), 0.0f, 1.0f) * alpha;
+        const float wgt = fmul(fclamp(fexp2(-F.m0_log2e * A), 0.0f, 1.0f), alpha);
         C.x = ffma(wgt, ffma(f, de.x, e0.x), C.x);
         C.y = ffma(wgt, ffma(f, de.y, e0.y), C.y);
         C.z = ffma(wgt, ffma(f, de.z, e0.z), C.z);
-        C.w += wgt;
+        C.w = fadd(C.w, wgt);   // not contracted with the product: as in blend_pair
         ++n;
     }
     __device__ __forceinline__ bool singular() const { return b0 > 0.0f && F.n == 0; }
@@ -518,11 +518,11 @@ struct PowerBlendBody {
         const float alpha = one_minus_exp_neg(a);
         const float z = warp_depth(t, wa, wb);
         const float A = power_fraction<N>(F, z, w0);
-        const float wgt = fclamp(fexp2(-F.m0_log2e * A), 0.0f, 1.0f) * alpha;
+        const float wgt = fmul(fclamp(fexp2(-F.m0_log2e * A), 0.0f, 1.0f), alpha);
         C.x = ffma(wgt, ffma(f, de.x, e0.x), C.x);
         C.y = ffma(wgt, ffma(f, de.y, e0.y), C.y);
         C.z = ffma(wgt, ffma(f, de.z, e0.z), C.z);
-        C.w += wgt;
+        C.w = fadd(C.w, wgt);   // not contracted with the product: as in blend_pair
         ++n;
     }
     __device__ __forceinline__ bool singular() const { return F.kind == kFrameFourMoments; }

@@ -122,15 +122,16 @@ MB_HD PowerFrame<N> make_power_frame(const float* m_in, float moment_bias) {
 // K(x, x) = sum_k (L^-1 v(x))_k^2 / D_k.
 template <int N, class T>
 MB_HD T power_kernel_diag(const PowerFrame<N>& P, T x) {
-    T y[N + 1], v = Vec<T>::splat(1.0f), K = Vec<T>::splat(0.0f);
+    T y[N + 1], v = x, K = Vec<T>::splat(P.invD[0]);   // y_0 = 1
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {
-        T t = v;
+    for (int i = 1; i <= N; ++i) {
+        const T l = Vec<T>::splat(-P.L[i * (i - 1) / 2]);
+        T t = i == 1 ? vadd(x, l) : vfma(v, x, l);      // x^i - L_i0
 #pragma unroll
-        for (int k = 0; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), y[k], t);
+        for (int k = 1; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), y[k], t);
         y[i] = t;
         K = vfma(vmul(t, t), Vec<T>::splat(P.invD[i]), K);
-        v = vmul(v, x);
+        if (i > 1 && i < N) v = vmul(v, x);
     }
     return K;
 }
@@ -150,16 +151,18 @@ MB_HD T power_weight(const PowerFrame<N>& P, T x0, T s) {
 template <int N, class T>
 MB_HD T power_fraction_generic(const PowerFrame<N>& P, T z0, float w0) {
     const T x0 = vfma(z0, Vec<T>::splat(P.inv_s), Vec<T>::splat(P.nmu));
-    T u[N + 1], y[N + 1], v = Vec<T>::splat(1.0f), K00 = Vec<T>::splat(0.0f);
+    T u[N + 1], y[N + 1], v = x0, K00 = Vec<T>::splat(P.invD[0]);   // u_0 = 1
+    y[0] = K00;
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {
-        T t = v;
+    for (int i = 1; i <= N; ++i) {
+        const T l = Vec<T>::splat(-P.L[i * (i - 1) / 2]);
+        T t = i == 1 ? vadd(x0, l) : vfma(v, x0, l);    // x0^i - L_i0
 #pragma unroll
-        for (int k = 0; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), u[k], t);
+        for (int k = 1; k < i; ++k) t = vfma(Vec<T>::splat(-P.L[i * (i - 1) / 2 + k]), u[k], t);
         u[i] = t;
         y[i] = vmul(t, Vec<T>::splat(P.invD[i]));
         K00 = vfma(t, y[i], K00);
-        v = vmul(v, x0);
+        if (i > 1 && i < N) v = vmul(v, x0);
     }
     // q = L^-T D^-1 y: coefficients of K(., x0) in the standardised frame
 #pragma unroll

@@ -45,6 +45,9 @@ MB_HD cv<T> cmul(cv<T> a, cv<T> b) {
 }
 template <class T>
 MB_HD cv<T> cconj(cv<T> a) { return {a.x, vneg(a.y)}; }
+// a - b
+template <class T>
+MB_HD cv<T> csub_of(cv<T> a, cf b) { return {vadd(a.x, Vec<T>::splat(-b.x)), vadd(a.y, Vec<T>::splat(-b.y))}; }
 // a - b * c
 template <class T>
 MB_HD cv<T> cfms(cv<T> a, cf b, cv<T> c) {
@@ -129,16 +132,17 @@ __device__ __forceinline__ void sincos_fast(float2 x, float2& sn, float2& cs) {
 template <int N, class T>
 MB_HD T trig_kernel_diag(const TrigFrame& F, cv<T> u) {
     cv<T> x[N + 1];
-    cv<T> ub = cconj(u), p = {Vec<T>::splat(1.0f), Vec<T>::splat(0.0f)};
-    T K = Vec<T>::splat(0.0f);
+    const cv<T> ub = cconj(u);
+    cv<T> p = ub;
+    T K = Vec<T>::splat(F.invD[0]);   // x_0 = 1
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {
-        cv<T> xi = p;
+    for (int i = 1; i <= N; ++i) {
+        cv<T> xi = csub_of(p, F.L[i * (i - 1) / 2]);
 #pragma unroll
-        for (int k = 0; k < i; ++k) xi = cfms(xi, F.L[i * (i - 1) / 2 + k], x[k]);
+        for (int k = 1; k < i; ++k) xi = cfms(xi, F.L[i * (i - 1) / 2 + k], x[k]);
         x[i] = xi;
         K = vfma(vfma(xi.x, xi.x, vmul(xi.y, xi.y)), Vec<T>::splat(F.invD[i]), K);
-        p = cmul(p, ub);
+        if (i < N) p = cmul(p, ub);
     }
     return K;
 }
@@ -146,10 +150,8 @@ MB_HD T trig_kernel_diag(const TrigFrame& F, cv<T> u) {
 // Weight of the node at s: 1 / K(u, u) at u = u0 (s + i) / (s - i).
 template <int N, class T>
 MB_HD T trig_weight(const TrigFrame& F, cv<T> u0, T s) {
-    const T one = Vec<T>::splat(1.0f);
-    const T s2 = vmul(s, s);
-    const T inv = vrcp(vadd(s2, one));
-    const cv<T> e = {vmul(vsub(s2, one), inv), vmul(vadd(s, s), inv)};
+    const T inv = vrcp(vfma(s, s, Vec<T>::splat(1.0f)));
+    const cv<T> e = {vmul(vfma(s, s, Vec<T>::splat(-1.0f)), inv), vmul(vtwice(s), inv)};
     return vrcp(trig_kernel_diag<N, T>(F, cmul(u0, e)));
 }
 
@@ -161,13 +163,13 @@ MB_HD T trig_weight(const TrigFrame& F, cv<T> u0, T s) {
 template <int N, class T, class W>
 MB_HD T front_weight(const T* r, Lanes<T> front, T rho0, T w0, const W& weight) {
     const T one = Vec<T>::splat(1.0f), zero = Vec<T>::splat(0.0f);
-    const T lo = vmul(w0, rho0), hi = vfma(vsub(w0, one), rho0, one);
+    const T hi = vfma(vsub(w0, one), rho0, one);
     // the side's outermost node, none where the other side holds all
     const T s = pick_gt(front, N / 2, r[N - 1], r[0]);
     T w = weight(s);
     w = pick_eq(front, 0, zero, pick_eq(front, N, zero, w));
     if (N == 4 && any_eq(front, 2)) w = vadd(w, pick_eq(front, 2, weight(r[1]), zero));
-    return pick_gt(front, N / 2, vsub(hi, w), vadd(lo, w));
+    return pick_gt(front, N / 2, vsub(hi, w), vfma(w0, rho0, w));
 }
 
 // Alg. 3 for trigonometric moments: fraction A of the optical depth in front
@@ -178,19 +180,19 @@ MB_HD T trig_fraction(const TrigFrame& F, const TrigTables& tab, T z0, float w0)
     sincos_fast(vmul(z0, Vec<T>::splat(tab.zone_scale)), u0.y, u0.x);
     // y = G^-1 w, w = conj(v(u0)) = (1, conj(u0), conj(u0)^2, ..)
     cv<T> w[N + 1], y[N + 1];
-    w[0] = {Vec<T>::splat(1.0f), Vec<T>::splat(0.0f)};
     w[1] = cconj(u0);
 #pragma unroll
     for (int k = 2; k <= N; ++k) w[k] = cmul(w[k - 1], w[1]);
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {
-        cv<T> t = w[i];
+    for (int i = 1; i <= N; ++i) {
+        cv<T> t = csub_of(w[i], F.L[i * (i - 1) / 2]);   // y_0 = 1
 #pragma unroll
-        for (int k = 0; k < i; ++k) t = cfms(t, F.L[i * (i - 1) / 2 + k], y[k]);
+        for (int k = 1; k < i; ++k) t = cfms(t, F.L[i * (i - 1) / 2 + k], y[k]);
         y[i] = t;
     }
+    y[0] = {Vec<T>::splat(F.invD[0]), Vec<T>::splat(0.0f)};
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {
+    for (int i = 1; i <= N; ++i) {
         const T d = Vec<T>::splat(F.invD[i]);
         y[i] = {vmul(y[i].x, d), vmul(y[i].y, d)};
     }
@@ -202,9 +204,11 @@ MB_HD T trig_fraction(const TrigFrame& F, const TrigTables& tab, T z0, float w0)
         y[i] = t;
     }
     // z_k = y_k u0^k; K(u0, u0) = Re sum z_k; real polynomial coefficients
-    T zr[N + 1], nzi[N + 1], K00 = Vec<T>::splat(0.0f);
+    T zr[N + 1], nzi[N + 1], K00 = y[0].x;
+    zr[0] = y[0].x;
+    nzi[0] = vneg(y[0].y);
 #pragma unroll
-    for (int k = 0; k <= N; ++k) {
+    for (int k = 1; k <= N; ++k) {
         const cv<T> z = cmul(y[k], cconj(w[k]));
         zr[k] = z.x;
         nzi[k] = vneg(z.y);
@@ -214,9 +218,9 @@ MB_HD T trig_fraction(const TrigFrame& F, const TrigTables& tab, T z0, float w0)
     T coef[N];
 #pragma unroll
     for (int m = 0; m < N; ++m) {
-        T acc = Vec<T>::splat(0.0f);
+        T acc = vfma(zr[0], Vec<T>::splat(tab.er[0][m]), vmul(nzi[0], Vec<T>::splat(tab.ei[0][m])));
 #pragma unroll
-        for (int k = 0; k <= N; ++k)
+        for (int k = 1; k <= N; ++k)
             acc = vfma(zr[k], Vec<T>::splat(tab.er[k][m]), vfma(nzi[k], Vec<T>::splat(tab.ei[k][m]), acc));
         coef[m] = vmul(acc, rho0);
     }

@@ -1,8 +1,11 @@
 // One value (float) or the values of two lattice points (float2) in the same
 // code: every helper is one operation with one rounding, on float2 one packed
 // FP32x2 instruction whose halves round as the scalar one, so that code
-// written with them gives a point the same bits alone and in a pair.  Also
-// the real roots of the monic cubics and quartics that the moment bounds
+// written with them gives a point the same bits alone and in a pair.  One
+// thing to keep to: the compiler may fuse a packed product that is used once
+// into a packed sum that takes it (the scalar intrinsics stay apart), so
+// every product that goes into a sum here is written as a vfma, and 2 x as
+// vtwice.  Also the real roots of the monic cubics and quartics that the moment bounds
 // meet, whose roots are all real.
 #pragma once
 #include "mboit_device.cuh"
@@ -22,6 +25,7 @@ MB_HD float vsub(float a, float b) { return fadd(a, -b); }
 MB_HD float vmul(float a, float b) { return fmul(a, b); }
 MB_HD float vfma(float a, float b, float c) { return ffma(a, b, c); }
 MB_HD float vneg(float a) { return -a; }
+MB_HD float vtwice(float a) { return fmul(a, 2.0f); }
 MB_HD float vmax(float a, float b) { return fmax_(a, b); }
 MB_HD float vmin(float a, float b) { return fmin_(a, b); }
 MB_HD float vrcp(float a) { return frcp(a); }
@@ -38,6 +42,7 @@ MB_V2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f),
 MB_V2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 MB_V2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 MB_V2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+MB_V2 vtwice(float2 a) { return __fmul2_rn(a, make_float2(2.0f, 2.0f)); }
 MB_V2 vmax(float2 a, float2 b) { return make_float2(fmax_(a.x, b.x), fmax_(a.y, b.y)); }
 MB_V2 vmin(float2 a, float2 b) { return make_float2(fmin_(a.x, b.x), fmin_(a.y, b.y)); }
 MB_V2 vrcp(float2 a) { return make_float2(frcp(a.x), frcp(a.y)); }
@@ -99,7 +104,7 @@ MB_HD T cos_third(T u) {
 template <class T>
 MB_HD T newton3(T a, T b, T c, T s) {
     const T f = vfma(vfma(vadd(s, a), s, b), s, c);
-    const T df = vfma(vfma(Vec<T>::splat(3.0f), s, vadd(a, a)), s, b);
+    const T df = vfma(vfma(Vec<T>::splat(3.0f), s, vtwice(a)), s, b);
     return vsub(s, vnonzero(df, vmul(f, vrcp(df))));
 }
 
@@ -109,10 +114,10 @@ template <class T>
 MB_HD void viete(T a, T b, T c, T& a3, T& m, T& cs) {
     a3 = vmul(a, Vec<T>::splat(1.0f / 3.0f));
     const T p = vfma(vneg(a), a3, b);
-    const T q = vfma(vfma(vadd(a3, a3), a3, vneg(b)), a3, c);   // 2 a3^3 - b a3 + c
+    const T q = vfma(vfma(vtwice(a3), a3, vneg(b)), a3, c);   // 2 a3^3 - b a3 + c
     const T pm = vmin(p, Vec<T>::splat(-1e-30f));
     const T h = vsqrt(vmul(pm, Vec<T>::splat(-1.0f / 3.0f)));
-    m = vadd(h, h);
+    m = vtwice(h);
     const T arg = vmul(vmul(Vec<T>::splat(3.0f), q), vrcp(vmul(pm, m)));
     cs = cos_third(vmax(vmin(arg, Vec<T>::splat(1.0f)), Vec<T>::splat(-1.0f)));
 }
@@ -151,9 +156,9 @@ MB_HD void quartic4(T a, T b, T c, T d, T r[4]) {
     T a3, am, cs;
     viete(p, rb, rc, a3, am, cs);
     const T m = vmax(newton3(p, rb, rc, vfma(am, cs, vneg(a3))), Vec<T>::splat(1e-30f));
-    const T m2 = vadd(m, m);
+    const T m2 = vtwice(m);
     const T sq = vsqrt(m2);
-    const T h = vfma(Vec<T>::splat(0.5f), p, m), g = vmul(q, vrcp(vadd(sq, sq)));
+    const T h = vfma(Vec<T>::splat(0.5f), p, m), g = vmul(q, vrcp(vtwice(sq)));
     // y^2 - sq y + (h + g) = 0 and y^2 + sq y + (h - g) = 0
     const T zero = Vec<T>::splat(0.0f), half = Vec<T>::splat(0.5f), four = Vec<T>::splat(-4.0f);
     const T d1 = vsqrt(vmax(vfma(four, vadd(h, g), m2), zero));
@@ -162,7 +167,7 @@ MB_HD void quartic4(T a, T b, T c, T d, T r[4]) {
     r[1] = vmul(half, vsub(d2, sq));
     r[2] = vmul(half, vsub(sq, d1));
     r[3] = vmul(half, vadd(sq, d1));
-    const T b2 = vadd(b, b), a3x = vmul(Vec<T>::splat(3.0f), a);
+    const T b2 = vtwice(b), a3x = vmul(Vec<T>::splat(3.0f), a);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const T s = vsub(r[i], a4);

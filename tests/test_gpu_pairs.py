@@ -31,7 +31,7 @@ def _clear_half(sc):
 SCENES = {
     "grid": lambda: scenes.blobs512(width=43, height=29, n_pieces=5, n=48),
     "grid_clear": lambda: _clear_half(scenes.blobs64(width=40, height=36)),
-    "grid_tiny": lambda: scenes.blobs512(width=9, height=5, n_pieces=2, n=17),
+    "grid_tiny": lambda: scenes.blobs512(width=9, height=5, n_pieces=2, n=33),
     "octree": lambda: scenes.amr_blobs(base=3, max_level=2, width=37, height=41, n_pieces=4),
     "mesh": lambda: scenes.tet_mesh(n=7, n_pieces=3, width=31, height=22),
 }
