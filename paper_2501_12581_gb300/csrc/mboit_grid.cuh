@@ -335,6 +335,25 @@ __device__ __forceinline__ bool blend_fused(const GridD& g, const uint8_t* __res
     return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body, NoStore{}, tma);
 }
 
+// The same for a tile whose rows found no room in the sample cache, as a call:
+// inlined it shares the registers of the loop over the cached rows, which
+// every other tile takes, and with trigonometric moments those spill.
+template <class Cfg, bool kSel, class Body>
+__device__ __noinline__ void blend_again(const GridD& g, const uint8_t* sel, float* win, const float* o_in,
+                                         const float* d_in, int k0, int k1, Body* body) {
+    const float o[3] = {o_in[0], o_in[1], o_in[2]}, d[3] = {d_in[0], d_in[1], d_in[2]};
+    blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, *body);
+}
+template <class Cfg, bool kSel, class Body>
+__device__ __forceinline__ void blend_uncached(const GridD& g, const uint8_t* sel, float* win, const float o_in[3],
+                                               const float d_in[3], int k0, int k1, Body& body) {
+    const float o[3] = {o_in[0], o_in[1], o_in[2]}, d[3] = {d_in[0], d_in[1], d_in[2]};
+    Body b = body;   // a copy: the caller's stays in registers
+    blend_again<Cfg, kSel>(g, sel, win, o, d, k0, k1, &b);
+    body.C = b.C;
+    body.n = b.n;
+}
+
 template <bool kSel, class Cfg, int MS, bool kCache = false>
 __global__ void __launch_bounds__(256, MS == 0 ? 5 : 1) k_pass1_fused(const __grid_constant__ GridD g, const float4* __restrict__ tf,
                                                      const uint8_t* __restrict__ sel, const __grid_constant__ ViewTable vt,
@@ -405,6 +424,8 @@ __global__ void __launch_bounds__(256) k_pass2_fused(const __grid_constant__ Gri
         if (kCache && tb >= 0) {
             const int kmin = __reduce_min_sync(0xffffffffu, k0), kmax = __reduce_max_sync(0xffffffffu, k1);
             blend_rows<kSel>(g, cache.vals + tb * 32, kmin, kmax, k0, k1, win, body);
+        } else if constexpr (kCache && (MS == 3 || MS == 4)) {
+            blend_uncached<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
         } else {
             blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);   // pass 2 has no TMA windows
         }

@@ -975,6 +975,27 @@ __device__ __forceinline__ void march_unit(const AmrD& a, const uint8_t* __restr
     }
 }
 
+// Pass 2 of a tile whose rows found no room in the sample cache: the march
+// again, as a call.  Inlined it shares the registers of the loop over the
+// cached rows, which every other tile takes: with trigonometric moments
+// those spill (1024^2 octree frame, 8 of them: 6.79 ms inlined, 6.55 ms as a
+// call).  The other sets fit inlined, and a call costs four moments 1 %.
+template <bool kSel, class V, class Body>
+__device__ __noinline__ void march_again(const V& a, const uint8_t* sel, const float* o_in, const float* d_in, int k0,
+                                         int k1, Body* body) {
+    const float o[3] = {o_in[0], o_in[1], o_in[2]}, d[3] = {d_in[0], d_in[1], d_in[2]};
+    march_unit<kSel>(a, sel, o, d, k0, k1, *body);
+}
+template <bool kSel, class V, class Body>
+__device__ __forceinline__ void march_uncached(const V& a, const uint8_t* sel, const float o_in[3], const float d_in[3],
+                                               int k0, int k1, Body& body) {
+    const float o[3] = {o_in[0], o_in[1], o_in[2]}, d[3] = {d_in[0], d_in[1], d_in[2]};
+    Body b = body;   // a copy: the caller's stays in registers
+    march_again<kSel>(a, sel, o, d, k0, k1, &b);
+    body.C = b.C;
+    body.n = b.n;
+}
+
 // Resident 256-thread blocks per SM the unit kernels are compiled for (the
 // walks and gathers are latency-bound: more warps hide more of it); the
 // trigonometric and 6-/8-power-moment bodies get 2, so that they keep their
@@ -1070,6 +1091,8 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 2>::value : 2) k_p
             else
                 blend_rows<RowsChecked<V, kSel>::value, false, kUnitRowChunk>(g, cache.vals + tb * 32, kmin, kmax, k0,
                                                                                k1, buf, body);
+        } else if constexpr (kCache && (MS == 3 || MS == 4)) {
+            march_uncached<kSel>(a, sel, o, d, k0, k1, body);
         } else {
             march_unit<kSel>(a, sel, o, d, k0, k1, body);
         }
