@@ -83,7 +83,9 @@ struct mboit_volume_s {
     uint32_t* d_bricks = nullptr;
     std::vector<int32_t> leaf_table;
     mb::TetD tet{};             // tetrahedral meshes: amr-like parameters plus the device tables below
-    int4* d_tcorners = nullptr;
+    int4* d_tcorners = nullptr;   // wide meshes
+    int4* d_tgeo = nullptr;       // narrow meshes: geometry and corner values per tet
+    float4* d_tval4 = nullptr;
     int4* d_tnbrs = nullptr;
     int4* d_tcells = nullptr;
     float* d_tcvals = nullptr;  // tile-row sample cache of the batched frame (grow only)
@@ -450,7 +452,8 @@ bool one_march(mboit_volume v, const std::vector<int32_t>& list, mb::SlotMap& ma
 // neighbours and the bin lists, after checking everything the exact
 // predicates rely on.
 struct TetHost {
-    std::vector<int4> verts, cells, nbrs, corners;
+    std::vector<int4> verts, cells, nbrs, corners, geo;
+    std::vector<float4> vals;
     bool narrow = false;
     std::vector<int32_t> bin_start, bin_tets;
     int32_t bdim[3] = {0, 0, 0};
@@ -588,9 +591,22 @@ mboit_status prepare_tets(const mboit_volume_desc* d, TetHost& h) {
         }
     }
     h.bin_start.assign(start.begin(), start.end());
-    h.corners.resize(4 * (size_t)nt);
+    if (h.narrow) {
+        h.geo.resize(4 * (size_t)nt);
+        h.vals.resize((size_t)nt);
+    } else {
+        h.corners.resize(4 * (size_t)nt);
+    }
     for (int64_t t = 0; t < nt; ++t) {
         const int4 c = h.cells[t];
+        if (h.narrow) {
+            const int4 v[4] = {h.verts[c.x], h.verts[c.y], h.verts[c.z], h.verts[c.w]};
+            mb::tet_geo(v, &h.geo[4 * (size_t)t]);
+            float x[4];
+            for (int i = 0; i < 4; ++i) std::memcpy(&x[i], &v[i].w, sizeof(float));
+            h.vals[(size_t)t] = make_float4(x[0], x[1], x[2], x[3]);
+            continue;
+        }
         h.corners[4 * t] = h.verts[c.x];
         h.corners[4 * t + 1] = h.verts[c.y];
         h.corners[4 * t + 2] = h.verts[c.z];
@@ -1056,7 +1072,12 @@ mboit_status mboit_create_volume(const mboit_volume_desc* d, mboit_volume* out) 
                 r = cudaMemcpy(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
             return r;
         };
-        e = up(v->d_tcorners, th.corners);
+        if (th.narrow) {
+            e = up(v->d_tgeo, th.geo);
+            if (e == cudaSuccess) e = up(v->d_tval4, th.vals);
+        } else {
+            e = up(v->d_tcorners, th.corners);
+        }
         if (e == cudaSuccess) e = up(v->d_tnbrs, th.nbrs);
         if (e == cudaSuccess) e = up(v->d_tcells, th.cells);
         if (e == cudaSuccess) e = up(v->d_bin_start, th.bin_start);
@@ -1065,6 +1086,8 @@ mboit_status mboit_create_volume(const mboit_volume_desc* d, mboit_volume* out) 
         mb::TetD& m = v->tet;
         m.g = g;
         m.corners = v->d_tcorners;
+        m.geo = v->d_tgeo;
+        m.vals = v->d_tval4;
         m.nbrs = v->d_tnbrs;
         m.narrow = th.narrow ? 1 : 0;
         m.n_tets = (int32_t)d->n_tets;
@@ -1113,6 +1136,8 @@ mboit_status mboit_destroy_volume(mboit_volume v) {
         cudaFree(v->d_fmap);
         cudaFree(v->d_bricks);
         cudaFree(v->d_tcorners);
+        cudaFree(v->d_tgeo);
+        cudaFree(v->d_tval4);
         cudaFree(v->d_tnbrs);
         cudaFree(v->d_tcells);
         cudaFree(v->d_tcvals);
@@ -1540,7 +1565,7 @@ mboit_status mboit_render_frame_host(mboit_volume v, const float* field_host, co
         if (v->kind == MBOIT_TET) {
             // vertex values live in the vertex records: stage, then scatter
             MB_CUDA(cudaMemcpyAsync(v->d_tvals, field_host, v->field_bytes, cudaMemcpyHostToDevice, s));
-            MB_CUDA(mb::launch_tet_values(v->d_tcorners, v->d_tcells, v->desc.n_tets, v->d_tvals, s));
+            MB_CUDA(mb::launch_tet_values(v->d_tcorners, v->d_tval4, v->d_tcells, v->desc.n_tets, v->d_tvals, s));
         } else {
             float* dst = const_cast<float*>(v->kind == MBOIT_AMR ? v->amr.values : v->grid.field);
             MB_CUDA(cudaMemcpyAsync(dst, field_host, v->field_bytes, cudaMemcpyHostToDevice, s));

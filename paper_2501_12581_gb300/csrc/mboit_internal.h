@@ -99,8 +99,10 @@ MB_HD uint32_t brick_word(int32_t leaf, int32_t shift) { return ((uint32_t)(127 
 // p * qscale.
 struct TetD {
     GridD g;
-    const int4* corners;       // per tet its 4 corners (positively oriented): snapped x, y, z and the
-                               //   value's float32 bits
+    const int4* corners;       // wide meshes: per tet its 4 corners (positively oriented), snapped x, y, z
+                               //   and the value's float32 bits
+    const int4* geo;           // narrow meshes: per tet 4 words of 16 bytes (tet_geo)
+    const float4* vals;        //   and its 4 corner values
     const int4* nbrs;          // per tet: the tet across the face opposite each corner (-1 on the boundary)
     const int32_t* bin_start;  // [nbins + 1]: bins of 2^bin_shift quanta, CSR over
     const int32_t* bin_tets;   //   the tets whose snapped bounding box meets the bin
@@ -243,8 +245,42 @@ cudaError_t launch_sortlast_march(bool fill, const TetD& m, const float4* tf, co
                                   int32_t n_slots, int32_t* counts, const int64_t* starts, int32_t* seg_key,
                                   float4* seg_col, cudaStream_t s);
 // Writes vertex values (values[vertex id]) into the .w words of the tets'
-// corner records.
-cudaError_t launch_tet_values(int4* corners, const int4* cells, int64_t n_tets, const float* values, cudaStream_t s);
+// corner records (wide meshes), or into their value records (narrow ones).
+cudaError_t launch_tet_values(int4* corners, float4* vals, const int4* cells, int64_t n_tets, const float* values,
+                              cudaStream_t s);
+
+// A narrow tet as the walk reads it: with corners v0..v3, the normals n1 =
+// (v2 - v0) x (v3 - v0), n2 = (v3 - v0) x (v1 - v0), n3 = (v1 - v0) x (v2 - v0) of
+// the faces opposite v1, v2, v3 (32 bits each), all through v0, and six times the
+// volume V.  At a point q, D_i = n_i . (q - v0), D_0 = V - D_1 - D_2 - D_3, and face
+// 0's normal is -(n1 + n2 + n3).  sh and inv serve the interpolation: the
+// smallest shift that brings V to 23 bits, and 1 / (V >> sh).
+//   geo[0] = (v0, sh)  geo[1] = (n1, V's low word)  geo[2] = (n2, its high word)  geo[3] = (n3, inv)
+inline void tet_geo(const int4 v[4], int4 geo[4]) {
+    int n[3][3], e[3][3];
+    for (int i = 0; i < 3; ++i) {
+        e[i][0] = v[i + 1].x - v[0].x;
+        e[i][1] = v[i + 1].y - v[0].y;
+        e[i][2] = v[i + 1].z - v[0].z;
+    }
+    for (int i = 0; i < 3; ++i) {
+        const int* a = e[(i + 1) % 3];
+        const int* b = e[(i + 2) % 3];
+        n[i][0] = a[1] * b[2] - a[2] * b[1];
+        n[i][1] = a[2] * b[0] - a[0] * b[2];
+        n[i][2] = a[0] * b[1] - a[1] * b[0];
+    }
+    const long long V = (long long)n[0][0] * e[0][0] + (long long)n[0][1] * e[0][1] + (long long)n[0][2] * e[0][2];
+    int sh = 0;
+    while ((V >> sh) >= (1 << 23)) ++sh;
+    const float inv = 1.0f / (float)(V >> sh);   // exact integer below 2^23, then one rounding
+    int bits;
+    __builtin_memcpy(&bits, &inv, sizeof bits);
+    geo[0] = make_int4(v[0].x, v[0].y, v[0].z, sh);
+    geo[1] = make_int4(n[0][0], n[0][1], n[0][2], (int)(uint32_t)V);
+    geo[2] = make_int4(n[1][0], n[1][1], n[1][2], (int)(V >> 32));
+    geo[3] = make_int4(n[2][0], n[2][1], n[2][2], bits);
+}
 
 // Table checks before a render's passes (failure detection): octree
 // finest-brick map entries are leaf ids or -1; mesh face neighbours are tet

@@ -88,10 +88,14 @@ cudaError_t launch_piece_kernel(const void* fn, const V& vol, const float4* tf, 
     return cudaLaunchKernel(fn, dim3(blocks > 0 ? blocks : 1), dim3(128), color ? args2 : args1, 0, s);
 }
 
-__global__ void k_tet_values(int4* __restrict__ corners, const int4* __restrict__ cells, int64_t n_tets,
-                             const float* __restrict__ values) {
+__global__ void k_tet_values(int4* __restrict__ corners, float4* __restrict__ vals, const int4* __restrict__ cells,
+                             int64_t n_tets, const float* __restrict__ values) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_tets; t += (int64_t)gridDim.x * blockDim.x) {
         const int4 c = cells[t];
+        if (vals) {
+            vals[t] = make_float4(values[c.x], values[c.y], values[c.z], values[c.w]);
+            continue;
+        }
         corners[4 * t].w = __float_as_int(values[c.x]);
         corners[4 * t + 1].w = __float_as_int(values[c.y]);
         corners[4 * t + 2].w = __float_as_int(values[c.z]);
@@ -330,9 +334,10 @@ cudaError_t launch_sortlast_march(bool fill, const TetD& m, const float4* tf, co
                                       seg_key, seg_col, s);
 }
 
-cudaError_t launch_tet_values(int4* corners, const int4* cells, int64_t n_tets, const float* values, cudaStream_t s) {
+cudaError_t launch_tet_values(int4* corners, float4* vals, const int4* cells, int64_t n_tets, const float* values,
+                              cudaStream_t s) {
     const int64_t nb = (n_tets + 255) / 256;
-    k_tet_values<<<(unsigned)(nb < 4096 ? (nb > 0 ? nb : 1) : 4096), 256, 0, s>>>(corners, cells, n_tets, values);
+    k_tet_values<<<(unsigned)(nb < 4096 ? (nb > 0 ? nb : 1) : 4096), 256, 0, s>>>(corners, vals, cells, n_tets, values);
     return cudaGetLastError();
 }
 

@@ -328,45 +328,61 @@ __device__ __forceinline__ void snap_point(const TetD& m, const float p[3], int 
     for (int c = 0; c < 3; ++c) q[c] = __float2int_rn(fmul(p[c], m.qscale));
 }
 
-// Sign of D for face (a, b) around `base` at q, D itself in D.  Narrow:
-// edges below 2^15 quanta, so the normal's components fit in 32 bits and D
-// is three 32 x 32 -> 64-bit multiply-adds.
-template <bool kNarrow>
+// Sign of D for face (a, b) around `base` at q, D itself in D (wide meshes).
 __device__ __forceinline__ bool face_positive(const int4 a, const int4 b, const int4 base, const int q[3],
                                               long long& D) {
     const int ax = a.x - base.x, ay = a.y - base.y, az = a.z - base.z;
     const int bx = b.x - base.x, by = b.y - base.y, bz = b.z - base.z;
     const int dx = q[0] - base.x, dy = q[1] - base.y, dz = q[2] - base.z;
-    long long nx, ny, nz;
-    if (kNarrow) {
-        const int n0 = ay * bz - az * by, n1 = az * bx - ax * bz, n2 = ax * by - ay * bx;
-        D = (long long)n0 * dx + (long long)n1 * dy + (long long)n2 * dz;
-        nx = n0;
-        ny = n1;
-        nz = n2;
-    } else {
-        nx = (long long)ay * bz - (long long)az * by;
-        ny = (long long)az * bx - (long long)ax * bz;
-        nz = (long long)ax * by - (long long)ay * bx;
-        D = nx * dx + ny * dy + nz * dz;
-    }
+    const long long nx = (long long)ay * bz - (long long)az * by;
+    const long long ny = (long long)az * bx - (long long)ax * bz;
+    const long long nz = (long long)ax * by - (long long)ay * bx;
+    D = nx * dx + ny * dy + nz * dz;
     if (D != 0) return D > 0;
     if (nx != 0) return nx > 0;
     if (ny != 0) return ny > 0;
     return nz > 0;
 }
 
+// Whether D, or if it is 0 the perturbed sign of its face's normal, is negative.
+__device__ __forceinline__ bool outside(long long D, int nx, int ny, int nz) {
+    if (D != 0) return D < 0;
+    return nx != 0 ? nx < 0 : ny != 0 ? ny < 0 : nz < 0;
+}
+
 // D_0..D_3 of q; returns -1 if q is inside, else a face that q lies
 // strictly outside of (the first one from `rot`, so that walks do not
-// always prefer one face).  Face `skip` (-1: none) is known to pass, its D
-// already in D[skip].
+// always prefer one face).  Wide meshes (v: the corners): face `skip` (-1:
+// none) is known to pass, its D already in D[skip].  Narrow ones (v: tet_geo):
+// edges below 2^15 quanta, so the stored normals fit in 32 bits and three
+// faces are three 32 x 32 -> 64-bit multiply-adds each, the fourth the
+// volume's remainder.  (From the corners a face cost six products, twelve
+// differences and those three multiply-adds; the walk waits on its loads and
+// its instructions about equally, and the record has the size the corners
+// had.)
 template <bool kNarrow>
 __device__ __forceinline__ int tet_exit_face(const int4 v[4], const int q[3], long long D[4], int rot, int skip) {
     unsigned out = 0;  // bit i: q is outside face i
-    if (skip != 0 && !face_positive<kNarrow>(v[2], v[1], v[3], q, D[0])) out |= 1u;
-    if (skip != 1 && !face_positive<kNarrow>(v[2], v[3], v[0], q, D[1])) out |= 2u;
-    if (skip != 2 && !face_positive<kNarrow>(v[3], v[1], v[0], q, D[2])) out |= 4u;
-    if (skip != 3 && !face_positive<kNarrow>(v[1], v[2], v[0], q, D[3])) out |= 8u;
+    if constexpr (kNarrow) {
+        const int dx = q[0] - v[0].x, dy = q[1] - v[0].y, dz = q[2] - v[0].z;
+#pragma unroll
+        for (int i = 1; i < 4; ++i)
+            D[i] = (long long)v[i].x * dx + (long long)v[i].y * dy + (long long)v[i].z * dz;
+        const long long V = ((long long)v[2].w << 32) | (unsigned)v[1].w;
+        D[0] = V - D[1] - D[2] - D[3];
+        out = (unsigned)(D[0] < 0) | (unsigned)(D[1] < 0) << 1 | (unsigned)(D[2] < 0) << 2 | (unsigned)(D[3] < 0) << 3;
+        if (D[0] == 0 || D[1] == 0 || D[2] == 0 || D[3] == 0) {
+            out = (unsigned)outside(D[0], -(v[1].x + v[2].x + v[3].x), -(v[1].y + v[2].y + v[3].y),
+                                    -(v[1].z + v[2].z + v[3].z));
+#pragma unroll
+            for (int i = 1; i < 4; ++i) out |= (unsigned)outside(D[i], v[i].x, v[i].y, v[i].z) << i;
+        }
+    } else {
+        if (skip != 0 && !face_positive(v[2], v[1], v[3], q, D[0])) out |= 1u;
+        if (skip != 1 && !face_positive(v[2], v[3], v[0], q, D[1])) out |= 2u;
+        if (skip != 2 && !face_positive(v[3], v[1], v[0], q, D[2])) out |= 4u;
+        if (skip != 3 && !face_positive(v[1], v[2], v[0], q, D[3])) out |= 8u;
+    }
     if (!out) return -1;
     rot &= 3;
     const unsigned r = ((out >> rot) | (out << (4 - rot))) & 15u;
@@ -388,22 +404,41 @@ __device__ __forceinline__ int bin_of(const TetD& m, const int q[3]) {
     return (b[2] * m.bdim[1] + b[1]) * m.bdim[0] + b[0];
 }
 
-// Per-ray walk state: the current tet, its neighbours and its corners
-// (snapped x, y, z, value bits).
+// Per-ray walk state: the current tet, its neighbours and its corners (wide:
+// snapped x, y, z, value bits) or its geometry record (narrow: tet_geo).
 struct TetWalk {
     int T = -1;
     int4 nb;
     int4 v[4];
 };
 
+template <bool kNarrow>
 __device__ __forceinline__ void load_tet(const TetD& m, int T, TetWalk& w) {
     w.T = T;
     w.nb = __ldg(m.nbrs + T);
-    const int4* c = m.corners + 4 * (size_t)T;
+    const int4* c = (kNarrow ? m.geo : m.corners) + 4 * (size_t)T;
     w.v[0] = __ldg(c);
     w.v[1] = __ldg(c + 1);
     w.v[2] = __ldg(c + 2);
     w.v[3] = __ldg(c + 3);
+}
+
+// Crosses face f of the walk's tet into its neighbour nt.  In a wide mesh the
+// entry face is then known to pass (its D is the exact negative of the exit
+// face's): `skip`.
+template <bool kNarrow>
+__device__ __forceinline__ void cross_face(const TetD& m, TetWalk& w, int f, int nt, long long D[4], int& skip) {
+    if constexpr (kNarrow) {
+        load_tet<true>(m, nt, w);
+    } else {
+        const int from = w.T;
+        const long long Df = f == 0 ? D[0] : f == 1 ? D[1] : f == 2 ? D[2] : D[3];
+        load_tet<false>(m, nt, w);
+        skip = w.nb.x == from ? 0 : w.nb.y == from ? 1 : w.nb.z == from ? 2 : 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (skip == i) D[i] = -Df;
+    }
 }
 
 // Tests the tets listed in q's bin one by one (the walk's fallback); on
@@ -414,7 +449,7 @@ __device__ __forceinline__ bool tet_search(const TetD& m, TetWalk& w, const int 
     bin_range(m, bin_of(m, q), j0, j1);
     for (int j = j0; j < j1; ++j) {
         TetWalk u;
-        load_tet(m, __ldg(m.bin_tets + j), u);
+        load_tet<kNarrow>(m, __ldg(m.bin_tets + j), u);
         if (tet_exit_face<kNarrow>(u.v, q, D, 0, -1) < 0) {
             w = u;
             return true;
@@ -437,7 +472,7 @@ __device__ __forceinline__ bool tet_walk(const TetD& m, TetWalk& w, const int q[
         int j0, j1;
         bin_range(m, b, j0, j1);
         if (j0 == j1) return false;  // no tet comes near q
-        load_tet(m, __ldg(m.bin_tets + j0), w);
+        load_tet<kNarrow>(m, __ldg(m.bin_tets + j0), w);
     }
     int skip = -1;
     for (int step = 0;; ++step) {
@@ -446,13 +481,7 @@ __device__ __forceinline__ bool tet_walk(const TetD& m, TetWalk& w, const int q[
         if (step + 1 >= m.max_walk) break;
         const int nt = pick(w.nb, f);
         if (nt < 0) break;
-        const int from = w.T;
-        const long long Df = f == 0 ? D[0] : f == 1 ? D[1] : f == 2 ? D[2] : D[3];
-        load_tet(m, nt, w);
-        skip = w.nb.x == from ? 0 : w.nb.y == from ? 1 : w.nb.z == from ? 2 : 3;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (skip == i) D[i] = -Df;
+        cross_face<kNarrow>(m, w, f, nt, D, skip);
     }
     return tet_search<kNarrow>(m, w, q, D);
 }
@@ -462,18 +491,33 @@ __device__ __forceinline__ float small_to_float(long long x) {
     return __int_as_float(0x4b000000 | (int)x) - 8388608.0f;
 }
 
-// Barycentric interpolation of the corner values: lambda_i = D_i / sum D.
-// Inside a tet every D_i >= 0; all four are shifted right together until
-// the sum fits in 23 bits, so each weight is off by at most 2^-23 and no
-// 64-bit conversion (a double-precision-pipe instruction) is needed.
-__device__ __forceinline__ float tet_value(const long long D[4], const int4 v[4]) {
-    const long long tot = D[0] + D[1] + D[2] + D[3];
-    const int sh = max(0, 41 - __clzll(tot));
-    const float inv = 1.0f / small_to_float(tot >> sh);
-    float s = small_to_float(D[0] >> sh) * __int_as_float(v[0].w);
-    s = ffma(small_to_float(D[1] >> sh), __int_as_float(v[1].w), s);
-    s = ffma(small_to_float(D[2] >> sh), __int_as_float(v[2].w), s);
-    s = ffma(small_to_float(D[3] >> sh), __int_as_float(v[3].w), s);
+// Barycentric interpolation of the corner values of the walk's tet: lambda_i =
+// D_i / sum D.  Inside a tet every D_i >= 0; all four are shifted right
+// together until the sum fits in 23 bits, so each weight is off by at most
+// 2^-23 and no 64-bit conversion (a double-precision-pipe instruction) is
+// needed.  The sum is the tet's volume: narrow meshes keep the shift and the
+// reciprocal with the tet.  Wide ones read the values (the .w words) again
+// here rather than keep them live through the walk.
+template <bool kNarrow>
+__device__ __forceinline__ float tet_value(const TetD& m, const TetWalk& w, const long long D[4]) {
+    float4 x;
+    int sh;
+    float inv;
+    if constexpr (kNarrow) {
+        x = __ldg(m.vals + w.T);
+        sh = w.v[0].w;
+        inv = __int_as_float(w.v[3].w);
+    } else {
+        const float* cw = reinterpret_cast<const float*>(m.corners + 4 * (size_t)w.T);
+        x = make_float4(__ldg(cw + 3), __ldg(cw + 7), __ldg(cw + 11), __ldg(cw + 15));
+        const long long tot = D[0] + D[1] + D[2] + D[3];
+        sh = max(0, 41 - __clzll(tot));
+        inv = 1.0f / small_to_float(tot >> sh);
+    }
+    float s = small_to_float(D[0] >> sh) * x.x;
+    s = ffma(small_to_float(D[1] >> sh), x.y, s);
+    s = ffma(small_to_float(D[2] >> sh), x.z, s);
+    s = ffma(small_to_float(D[3] >> sh), x.w, s);
     return s * inv;
 }
 
@@ -491,7 +535,7 @@ __device__ __forceinline__ bool piece_sample(const TetT<kNarrow>& m, const int32
     long long D[4];
     if (!tet_walk<kNarrow>(m, w, q, D)) return false;
     if (__ldg(pou + w.T) != piece) return false;
-    val = tf_x(g, tet_value(D, w.v));
+    val = tf_x(g, tet_value<kNarrow>(m, w, D));
     return true;
 }
 
@@ -501,70 +545,69 @@ __device__ __forceinline__ bool piece_sample(const TetT<kNarrow>& m, const int32
 // finest-brick map, its value from the leaf's own vertex block.  Mesh: the
 // tet comes from a walk that starts at the previous sample's tet.
 
-// Batched march over a mesh.  One iteration is one tet test for every lane
-// of the warp: it either places the current lattice point (the sample is
-// taken, the next point comes up) or crosses a face towards it, so the
-// lanes stay together in the test and part only for the sample or the
-// crossing.  The owners are those of tet_walk: the same walk, the same
-// fallback.  `store` gets every lattice point's value (NaN: not sampled).
+// Batched march over a mesh, in lockstep: the warp takes the lattice rows one
+// by one, every lane inside its own [k0, k1] crosses faces from its previous
+// point's tet until the new point is inside, and the lanes sample together.
+// (One loop of tet tests, each lane on its own row, sampled a few lanes at a
+// time: 18 of 32 lanes active.)  The owners are those of tet_walk: the same
+// walk, the same fallback.  `store` gets every lattice point's value (NaN: not
+// sampled).  With zrows (a warp's DepthRows) the moments take the rows' shared
+// depth powers.
 template <bool kSel, class Body, bool kNarrow, class Store = NoStore>
 __device__ __forceinline__ void march_unit(const TetT<kNarrow>& m, const uint8_t* __restrict__ sel, const float o[3],
-                                           const float d[3], int k0, int k1, Body& body, Store store = Store{}) {
+                                           const float d[3], int k0, int k1, Body& body, Store store = Store{},
+                                           float4* zrows = nullptr) {
+    constexpr bool kRows = std::is_same<Body, MomentBody>::value;
     const GridD& g = m.g;
-    if (k0 > k1) return;
-    store.seek(k0);
-    const float tz = lattice_t(k1, g.step);
-    float t = lattice_t(k0, g.step);
-    int q[3];
-    {
-        const float p[3] = {ffma(t, d[0], o[0]), ffma(t, d[1], o[1]), ffma(t, d[2], o[2])};
-        snap_point(m, p, q);
-    }
+    const unsigned full = 0xffffffffu;
+    const bool any = k0 <= k1;
+    const int kmin = __reduce_min_sync(full, any ? k0 : 0x7fffffff);
+    const int kmax = __reduce_max_sync(full, any ? k1 : -1);
+    if (any) store.seek(k0);
     TetWalk w;
-    {
-        const int b = bin_of(m, q);
-        int j0, j1;
-        bin_range(m, b, j0, j1);
-        if (j0 < j1) load_tet(m, __ldg(m.bin_tets + j0), w);
-    }
-    long long D[4];
-    int skip = -1, steps = 0;
-    while (t <= tz) {
-        const int f = w.T >= 0 ? tet_exit_face<kNarrow>(w.v, q, D, steps, skip) : -2;
-        if (f >= 0) {
-            const int nt = pick(w.nb, f);
-            if (nt >= 0 && steps + 1 < m.max_walk) {
-                const int from = w.T;
-                const long long Df = f == 0 ? D[0] : f == 1 ? D[1] : f == 2 ? D[2] : D[3];
-                load_tet(m, nt, w);
-                skip = w.nb.x == from ? 0 : w.nb.y == from ? 1 : w.nb.z == from ? 2 : 3;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (skip == i) D[i] = -Df;
-                ++steps;
-                continue;
-            }
+    for (int k = kmin; k <= kmax; ++k) {
+        if constexpr (kRows) {
+            if (zrows && ((k - kmin) & (kDepthRows - 1)) == 0) DepthRows{zrows}.fill(k, g.step, body.wa, body.wb);
         }
-        const bool found = f == -1 || tet_search<kNarrow>(m, w, q, D);
-        float val = __int_as_float(0x7fc00000);
+        if (k < k0 || k > k1) continue;
+        const float t = lattice_t(k, g.step);
+        const float p[3] = {ffma(t, d[0], o[0]), ffma(t, d[1], o[1]), ffma(t, d[2], o[2])};
+        int q[3];
+        snap_point(m, p, q);
+        if (w.T < 0) {
+            int j0, j1;
+            bin_range(m, bin_of(m, q), j0, j1);
+            if (j0 < j1) load_tet<kNarrow>(m, __ldg(m.bin_tets + j0), w);
+        }
+        long long D[4];
+        bool found = false;
+        if (w.T >= 0) {
+            int skip = -1, f;
+            for (int steps = 0;; ++steps) {
+                f = tet_exit_face<kNarrow>(w.v, q, D, steps, skip);
+                if (f < 0 || steps + 1 >= m.max_walk) break;
+                const int nt = pick(w.nb, f);
+                if (nt < 0) break;
+                cross_face<kNarrow>(m, w, f, nt, D, skip);
+            }
+            found = f < 0;
+        }
+        if (!found) found = tet_search<kNarrow>(m, w, q, D);
         bool take = found && (!kSel || __ldg(sel + w.T));
         if constexpr (TakesUnits<Body>::value) take = take && body.enter(w.T);
         if (take) {
-            // the corner values (the .w words) read again here rather than
-            // kept live through the walk, which only tests x, y, z: fewer
-            // spilled registers in the loop (the same bits, so the same value)
-            const int* cw = reinterpret_cast<const int*>(m.corners + 4 * (size_t)w.T);
-            const int4 vw[4] = {make_int4(0, 0, 0, __ldg(cw + 3)), make_int4(0, 0, 0, __ldg(cw + 7)),
-                                make_int4(0, 0, 0, __ldg(cw + 11)), make_int4(0, 0, 0, __ldg(cw + 15))};
-            val = tf_x(g, tet_value(D, vw));
+            const float val = tf_x(g, tet_value<kNarrow>(m, w, D));
+            store.put(val);
+            if constexpr (kRows) {
+                if (zrows) {
+                    body.add(val, 1.0f, zrows[(k - kmin) & (kDepthRows - 1)]);
+                    continue;
+                }
+            }
             body(t, val);
+        } else {
+            store.put(__int_as_float(0x7fc00000));
         }
-        store.put(val);
-        t += g.step;
-        const float p[3] = {ffma(t, d[0], o[0]), ffma(t, d[1], o[1]), ffma(t, d[2], o[2])};
-        snap_point(m, p, q);
-        skip = -1;
-        steps = 0;
     }
 }
 
@@ -1041,9 +1084,9 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 1>::value : 2) k_p
             }
         } else if constexpr (kCache) {
             RowStore st{tile_rows(cache, ctr, tile, k0, k1)};
-            march_unit<kSel>(a, sel, o, d, k0, k1, body, st);
+            march_unit<kSel>(a, sel, o, d, k0, k1, body, st, zrows);
         } else {
-            march_unit<kSel>(a, sel, o, d, k0, k1, body);
+            march_unit<kSel>(a, sel, o, d, k0, k1, body, NoStore{}, zrows);
         }
         if (valid) body.store(g, moments, S, S.moment_off, py * S.v.width + px);
         warp_add_u64(&ctr->samples[0], body.n);
