@@ -271,8 +271,8 @@ inline void tet_geo(const int4 v[4], int4 geo[4]) {
         n[i][2] = a[0] * b[1] - a[1] * b[0];
     }
     const long long V = (long long)n[0][0] * e[0][0] + (long long)n[0][1] * e[0][1] + (long long)n[0][2] * e[0][2];
-    int sh = 0;
-    while ((V >> sh) >= (1 << 23)) ++sh;
+    const int bits_of = 64 - __builtin_clzll((unsigned long long)V);   // V > 0
+    const int sh = bits_of > 23 ? bits_of - 23 : 0;
     const float inv = 1.0f / (float)(V >> sh);   // exact integer below 2^23, then one rounding
     int bits;
     __builtin_memcpy(&bits, &inv, sizeof bits);
