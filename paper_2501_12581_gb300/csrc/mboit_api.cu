@@ -208,6 +208,14 @@ mboit_status convert_tf(const mboit_volume_desc* d, float4* tf) {
     return MBOIT_OK;
 }
 
+// kFlagThin where every entry's absorbance of one step is below 1/4 (a linear
+// interpolation of entries then is too).
+uint32_t thin_flag(const float4* tf) {
+    float most = 0.0f;
+    for (int j = 0; j < 256; ++j) most = std::max(most, tf[j].w);
+    return most < 0.25f ? mb::kFlagThin : 0u;
+}
+
 // Grid geometry and sampling parameters of a descriptor (validated).
 void fill_grid(const mboit_volume_desc* d, mb::GridD& g) {
     const int B = 1 << d->brick_log2;
@@ -977,6 +985,7 @@ mboit_status mboit_create_volume(const mboit_volume_desc* d, mboit_volume* out) 
     mb::GridD& g = v->grid;
     fill_grid(d, g);
     fill_trig(g.trig, d->moment_set, d->storage, d->moment_bias);
+    g.flags |= thin_flag(tf.data());
     v->nbricks = (int64_t)g.nbx * g.nby * g.nbz;
     v->field_bytes = (size_t)g.nx * g.ny * g.nz * sizeof(float);
     v->kind = d->kind;

@@ -68,6 +68,21 @@ __device__ __forceinline__ bool field_sample(const GridD& g, const uint8_t* __re
     return true;
 }
 
+// Whole part (as table or cell index) and fraction of two coordinates in [0,
+// 2^23) at once: adding 2^23 rounding down leaves the whole part in the low
+// mantissa bits.  Equal to (int)x and x - (float)(int)x; the conversions it
+// replaces share a slower pipe.
+struct Split2 {
+    float2 f;
+    int a, b;   // carry the bits of 2^23 (kSplitBias)
+};
+constexpr int kSplitBias = 0x4b000000;
+__device__ __forceinline__ Split2 split2(float2 x) {
+    const float2 m = __fadd2_rd(x, make_float2(8388608.0f, 8388608.0f));
+    const float2 w = __fadd2_rn(m, make_float2(-8388608.0f, -8388608.0f));
+    return {__ffma2_rn(w, make_float2(-1.0f, -1.0f), x), __float_as_int(m.x), __float_as_int(m.y)};
+}
+
 // Transfer-function table coordinate of sample value v (O5): the value
 // normalised to [0, 1] by the table's range, times 255, clamped.  The
 // marches hand this to the per-sample bodies, and the frame's sample cache
@@ -190,6 +205,28 @@ struct MomentBody {
         m34 = __ffma2_rn(aa, make_float2(zp.z, zp.w), m34);
         ++n;
     }
+    // Two points in a row (weight 1): equal to two calls of add, bit for bit.
+    // Where ok is false a point adds nothing.
+    __device__ __forceinline__ void add2(float xa, float xb, bool oka, bool okb, float4 za, float4 zb) {
+        const Split2 s = split2(make_float2(xa, xb));
+        const float2 ea = s_sig[s.a - kSplitBias], eb = s_sig[s.b - kSplitBias];
+        const float a = oka ? fmin_(ffma(s.f.x, ea.y, ea.x), amax) : 0.0f;
+        const float b = okb ? fmin_(ffma(s.f.y, eb.y, eb.x), amax) : 0.0f;
+        m0 += a;
+        m12 = __ffma2_rn(make_float2(a, a), make_float2(za.x, za.y), m12);
+        m34 = __ffma2_rn(make_float2(a, a), make_float2(za.z, za.w), m34);
+        m0 += b;
+        m12 = __ffma2_rn(make_float2(b, b), make_float2(zb.x, zb.y), m12);
+        m34 = __ffma2_rn(make_float2(b, b), make_float2(zb.z, zb.w), m34);
+        n += (unsigned)oka + (unsigned)okb;
+    }
+    // The same with the depth powers of lattice depths ta and tb (depth_powers).
+    __device__ __forceinline__ void pair(float ta, float tb, float xa, float xb, bool oka, bool okb) {
+        const float2 l = __ffma2_rn(make_float2(flog2(ta), flog2(tb)), make_float2(wa, wa), make_float2(wb, wb));
+        const float2 z = make_float2(fclamp(l.x, -1.0f, 1.0f), fclamp(l.y, -1.0f, 1.0f));
+        const float2 z2 = __fmul2_rn(z, z), z3 = __fmul2_rn(z2, z), z4 = __fmul2_rn(z3, z);
+        add2(xa, xb, oka, okb, make_float4(z.x, z2.x, z3.x, z4.x), make_float4(z.y, z2.y, z3.y, z4.y));
+    }
     __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) {
         add(xt, ws, depth_powers(t, wa, wb));
     }
@@ -218,15 +255,15 @@ struct DepthRows {
 // taken for a, then b, so that the result equals two one-point calls bit for
 // bit.  A point with ok = false adds nothing: its table coordinate is replaced
 // by 0 (no NaN enters) and its weight by 0, and fma(0, c, C) = C.  `live` false:
-// the pixel has no absorbance and its T may be NaN; nothing is added.  T():
-// both transmittances.
+// the pixel has no absorbance and its T may be NaN; nothing is added.  `thin`:
+// no absorbance reaches 1/4 (kFlagThin).  transmittances(): both T.
 template <class T>
 __device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float4& C, unsigned& n, float xa, float xb,
-                                           bool oka, bool okb, bool live, unsigned act, const T& transmittances) {
-    xa = oka ? xa : 0.0f;
-    xb = okb ? xb : 0.0f;
-    const int ia = (int)xa, ib = (int)xb;
-    const float fa = xa - (float)ia, fb = xb - (float)ib;
+                                           bool oka, bool okb, bool live, bool thin, unsigned act,
+                                           const T& transmittances) {
+    const Split2 x = split2(make_float2(oka ? xa : 0.0f, okb ? xb : 0.0f));
+    const int ia = x.a - kSplitBias, ib = x.b - kSplitBias;
+    const float fa = x.f.x, fb = x.f.y;
     const float4 ea = s_tf[2 * ia], da = s_tf[2 * ia + 1], eb = s_tf[2 * ib], db = s_tf[2 * ib + 1];
     // the table lerps as pairs: (r, g) and (b, absorbance) of each point
     const float2 rga = __ffma2_rn(make_float2(fa, fa), make_float2(da.x, da.y), make_float2(ea.x, ea.y));
@@ -242,7 +279,7 @@ __device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float
     p = __ffma2_rn(a, p, make_float2(-0.5f, -0.5f));
     p = __ffma2_rn(a, p, make_float2(1.0f, 1.0f));
     float2 alpha = __fmul2_rn(a, p);
-    if (__any_sync(act, a.x >= 0.25f || a.y >= 0.25f)) {
+    if (!thin && __any_sync(act, a.x >= 0.25f || a.y >= 0.25f)) {
         const float2 ng = __fmul2_rn(a, make_float2(-kLog2e, -kLog2e));
         const float2 dir = __ffma2_rn(make_float2(fexp2(ng.x), fexp2(ng.y)), make_float2(-1.0f, -1.0f),
                                       make_float2(1.0f, 1.0f));
@@ -266,6 +303,7 @@ struct BlendBody {
     Frame F;
     float tf_scale, tf_bias, amax, wa, wb, w0;
     float b0;
+    bool thin;            // kFlagThin
     float4 C = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     unsigned n = 0;
     bool fp64 = false;    // the frame was set up in FP64 (near-singular Hankel matrix)
@@ -294,7 +332,7 @@ struct BlendBody {
     __device__ __forceinline__ bool pairs() const { return F.kind == kFrameGeneric || F.kind == kFrameEmpty; }
     // Two points of a generic frame: equal to two sample<true> calls bit for bit.
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, true, act, [&]() {
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, true, thin, act, [&]() {
             const float2 ex = __fmul2_rn(make_float2(-F.m0_log2e, -F.m0_log2e), bound_generic2(F, z, w0, act));
             return make_float2(fexp2(ex.x), fexp2(ex.y));
         });
@@ -420,6 +458,7 @@ struct TrigBlendBody {
     TrigFrame F;
     float tf_scale, tf_bias, amax, wa, wb, w0;
     float b0;
+    bool thin;            // kFlagThin
     float4 C = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     unsigned n = 0;
     __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) {
@@ -441,7 +480,7 @@ struct TrigBlendBody {
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
     __device__ __forceinline__ bool pairs() const { return !singular(); }
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.n != 0, act,
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.n != 0, thin, act,
                    [&]() { return heavy_transmittance(F.m0_log2e, trig_fraction<N, float2>(F, *T, z, w0)); });
     }
 };
@@ -508,6 +547,7 @@ struct PowerBlendBody {
     PowerFrame<N> F;
     float tf_scale, tf_bias, amax, wa, wb, w0;
     float b0;
+    bool thin;            // kFlagThin
     float4 C = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     unsigned n = 0;
     __device__ __forceinline__ void operator()(float t, float xt, float ws = 1.0f) {
@@ -529,7 +569,7 @@ struct PowerBlendBody {
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
     __device__ __forceinline__ bool pairs() const { return !singular(); }
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.kind == kFrameGeneric, act,
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.kind == kFrameGeneric, thin, act,
                    [&]() { return heavy_transmittance(F.m0_log2e, power_fraction_generic<N, float2>(F, z, w0)); });
     }
 };
@@ -586,6 +626,7 @@ __device__ __forceinline__ BlendBody blend_body_of(const float4* s_tf, const Gri
     b.wa = S.v.warp_a;
     b.wb = S.v.warp_b;
     b.w0 = g.overestimation;
+    b.thin = (g.flags & kFlagThin) != 0;
     const float m[5] = {valid ? mb.m0 : 0.0f, valid ? mb.m12.x : 0.0f, valid ? mb.m12.y : 0.0f,
                         valid ? mb.m34.x : 0.0f, valid ? mb.m34.y : 0.0f};
     b.F = pixel_frame(g, m, &b.fp64);
@@ -606,6 +647,7 @@ __device__ __forceinline__ typename Bodies<MS>::Blend make_blend_body(const floa
     b.wa = S.v.warp_a;
     b.wb = S.v.warp_b;
     b.w0 = g.overestimation;
+    b.thin = (g.flags & kFlagThin) != 0;
     if constexpr (MS == 0) {
         float m[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         if (valid) load_moments(moments, S, off, pix, m);

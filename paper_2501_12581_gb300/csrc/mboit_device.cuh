@@ -116,8 +116,22 @@ MB_HD float fdiv_fast(float a, float b) {
 #endif
 }
 MB_HD float frcp(float x) { return fdiv_fast(1.0f, x); }
-MB_HD float fmin_(float a, float b) { return a < b ? a : b; }
-MB_HD float fmax_(float a, float b) { return a > b ? a : b; }
+// the second operand where the first is NaN (a limit, never NaN); on the
+// device one instruction, where the comparison and select are two
+MB_HD float fmin_(float a, float b) {
+#if defined(__CUDA_ARCH__)
+    return fminf(a, b);
+#else
+    return a < b ? a : b;
+#endif
+}
+MB_HD float fmax_(float a, float b) {
+#if defined(__CUDA_ARCH__)
+    return fmaxf(a, b);
+#else
+    return a > b ? a : b;
+#endif
+}
 MB_HD float fclamp(float x, float lo, float hi) { return fmin_(fmax_(x, lo), hi); }
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -148,6 +162,9 @@ struct TrigTables {
 constexpr uint32_t kFlagRawSum = 0x1u;
 constexpr uint32_t kFlagAdaptiveStep = 0x4u;
 constexpr uint32_t kFlagFp64Setup = 0x8u;   // every pixel's frame set up in FP64
+// Set by the library: every table entry's absorbance of one step is below 1/4,
+// so a fixed-step sample's opacity always takes the series (one_minus_exp_neg).
+constexpr uint32_t kFlagThin = 0x40000000u;
 // Test hook of the TMA wait limit (set by mboit_debug_corrupt, never by a
 // descriptor): window loads arm their barrier but issue no copy.
 constexpr uint32_t kFlagDebugNoCopy = 0x80000000u;

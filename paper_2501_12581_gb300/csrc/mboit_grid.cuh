@@ -251,25 +251,56 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
             const float tz = lattice_t(kz, g.step);
             store.seek(ka);
             float t0 = lattice_t(ka, g.step);
-            if constexpr (!kSel && !TakesUnits<Body>::value) {
-                // two points at a time: both positions, then both points' 16
+            if constexpr (!TakesUnits<Body>::value) {
+                // two points at a time: both positions, whole parts and
+                // fractions as packed FP32x2 operations, then both points' 16
                 // window reads, then the store and the body in order
-                auto window_value = [&](float t) {
-                    const float p0 = ffma(t, d[0], o[0]), p1 = ffma(t, d[1], o[1]), p2 = ffma(t, d[2], o[2]);
-                    const int ix = (int)p0, iy = (int)p1, iz = (int)p2;
-                    const float* c = wbase + iz * Cfg::Plane + iy * Cfg::Pitch + ix;
-                    return tf_x(g, trilinear8(c[0], c[1], c[Cfg::Pitch], c[Cfg::Pitch + 1], c[Cfg::Plane],
-                                              c[Cfg::Plane + 1], c[Cfg::Plane + Cfg::Pitch],
-                                              c[Cfg::Plane + Cfg::Pitch + 1], p0 - (float)ix, p1 - (float)iy,
-                                              p2 - (float)iz));
-                };
+                const float2 o0 = make_float2(o[0], o[0]), o1 = make_float2(o[1], o[1]), o2 = make_float2(o[2], o[2]);
+                const float2 d0 = make_float2(d[0], d[0]), d1 = make_float2(d[1], d[1]), d2 = make_float2(d[2], d[2]);
+                // the window's origin, and the bits that split2's whole parts carry (mod 2^32)
+                const int base = (LO[2] + kSplitBias) * Cfg::Plane + (LO[1] + kSplitBias) * Cfg::Pitch + LO[0] + kSplitBias;
                 for (; t0 + g.step <= tz; t0 += 2.0f * g.step) {
                     const float tb = t0 + g.step;
-                    const float xa = window_value(t0), xb = window_value(tb);
-                    store.put(xa);
-                    body(t0, xa);
-                    store.put(xb);
-                    body(tb, xb);
+                    const float2 t2 = make_float2(t0, tb);
+                    const Split2 x = split2(__ffma2_rn(t2, d0, o0)), y = split2(__ffma2_rn(t2, d1, o1)),
+                                 z = split2(__ffma2_rn(t2, d2, o2));
+                    bool oka = true, okb = true;
+                    if constexpr (kSel) {
+                        auto wanted = [&](int ix, int iy, int iz) {
+                            const int bx = (ix - kSplitBias) >> g.brick_log2, by = (iy - kSplitBias) >> g.brick_log2,
+                                      bz = (iz - kSplitBias) >> g.brick_log2;
+                            return __ldg(sel + (bz * g.nby + by) * g.nbx + bx) != 0;
+                        };
+                        oka = wanted(x.a, y.a, z.a);
+                        okb = wanted(x.b, y.b, z.b);
+                        if (!__any_sync(__activemask(), oka || okb)) {   // bricks that no lane wants
+                            store.put(__int_as_float(0x7fc00000));
+                            store.put(__int_as_float(0x7fc00000));
+                            continue;
+                        }
+                    }
+                    const float* ca = win + (z.a * Cfg::Plane + y.a * Cfg::Pitch + x.a - base);
+                    const float* cb = win + (z.b * Cfg::Plane + y.b * Cfg::Pitch + x.b - base);
+                    auto at = [&](int k) { return make_float2(ca[k], cb[k]); };
+                    auto lerp = [](float2 f, float2 v0, float2 v1) { return __ffma2_rn(f, fsub2(v1, v0), v0); };
+                    const float2 lo = lerp(y.f, lerp(x.f, at(0), at(1)), lerp(x.f, at(Cfg::Pitch), at(Cfg::Pitch + 1)));
+                    const float2 hi = lerp(y.f, lerp(x.f, at(Cfg::Plane), at(Cfg::Plane + 1)),
+                                           lerp(x.f, at(Cfg::Plane + Cfg::Pitch), at(Cfg::Plane + Cfg::Pitch + 1)));
+                    const float2 v = __ffma2_rn(lerp(z.f, lo, hi), make_float2(g.tf_scale, g.tf_scale),
+                                                make_float2(g.tf_bias, g.tf_bias));
+                    const float xa = fclamp(v.x, 0.0f, 255.0f), xb = fclamp(v.y, 0.0f, 255.0f);
+                    store.put(oka ? xa : __int_as_float(0x7fc00000));
+                    if constexpr (std::is_same<Body, MomentBody>::value) {
+                        store.put(okb ? xb : __int_as_float(0x7fc00000));
+                        body.pair(t0, tb, xa, xb, oka, okb);
+                    } else if constexpr (HasPair<Body>::value) {
+                        store.put(okb ? xb : __int_as_float(0x7fc00000));
+                        body.pair(make_float2(body.depth(t0), body.depth(tb)), xa, xb, oka, okb, __activemask());
+                    } else {
+                        if (oka) body(t0, xa);
+                        store.put(okb ? xb : __int_as_float(0x7fc00000));
+                        if (okb) body(tb, xb);
+                    }
                 }
             }
             for (float t = t0; t <= tz; t += g.step) {
@@ -319,18 +350,15 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
 }
 
 
-// Pass 2 marching the field: with four power moments, a warp whose lanes
-// with samples all have a generic frame takes the body without the
-// per-sample test of the frame's kind (the same arithmetic and result).
+// Pass 2 marching the field, two points at a time in a warp whose lanes with
+// samples all may (pairs()): the same bits.
 template <class Cfg, bool kSel, class Body>
 __device__ __forceinline__ bool blend_fused(const GridD& g, const uint8_t* __restrict__ sel, float* __restrict__ win,
                                             const float o[3], const float d[3], int k0, int k1, Body& body,
                                             TmaWin* tma = nullptr) {
-    if constexpr (std::is_same<Body, BlendBody>::value) {
-        if (__all_sync(0xffffffffu, k0 > k1 || body.F.kind == kFrameGeneric)) {
-            PairBlend<BlendBody> gb{body};
-            return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, gb, NoStore{}, tma);
-        }
+    if (__all_sync(0xffffffffu, k0 > k1 || body.pairs())) {
+        PairBlend<Body> pb{body};
+        return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, pb, NoStore{}, tma);
     }
     return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body, NoStore{}, tma);
 }
@@ -355,7 +383,7 @@ __device__ __forceinline__ void blend_uncached(const GridD& g, const uint8_t* se
 }
 
 template <bool kSel, class Cfg, int MS, bool kCache = false>
-__global__ void __launch_bounds__(256, MS == 0 ? 5 : 1) k_pass1_fused(const __grid_constant__ GridD g, const float4* __restrict__ tf,
+__global__ void __launch_bounds__(256, 4) k_pass1_fused(const __grid_constant__ GridD g, const float4* __restrict__ tf,
                                                      const uint8_t* __restrict__ sel, const __grid_constant__ ViewTable vt,
                                                      char* __restrict__ moments, Counters* __restrict__ ctr,
                                                      const TileCache cache, const __grid_constant__ CUtensorMap tmap) {
@@ -426,6 +454,10 @@ __global__ void __launch_bounds__(256) k_pass2_fused(const __grid_constant__ Gri
             blend_rows<kSel>(g, cache.vals + tb * 32, kmin, kmax, k0, k1, win, body);
         } else if constexpr (kCache && (MS == 3 || MS == 4)) {
             blend_uncached<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
+        } else if constexpr (kCache) {
+            // a tile whose rows found no room: one point at a time, so that
+            // this rare march takes no registers from the loop over the rows
+            march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
         } else {
             blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);   // pass 2 has no TMA windows
         }

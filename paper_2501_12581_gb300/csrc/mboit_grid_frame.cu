@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) k_frame_fused(const __grid_constant__ Gri
         if (base >= 0)
             blend_rows<kSel>(g, cache.vals + base * 32, kmin, kmax, k0, k1, win, body);
         else
-            if (!blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body, &tw)) return;
+            if (!march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body, NoStore{}, &tw)) return;   // no room in the cache
         if (valid) {
             float4* out = reinterpret_cast<float4*>(color + S.color_off) + pix;
             if (mode == kColorResolved)

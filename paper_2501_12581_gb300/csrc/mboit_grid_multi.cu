@@ -8,14 +8,14 @@
 // memory); their fields, domains, sampling steps and moment parameters are
 // their own, read from the GridTable kernel parameter by the view's index.
 // The per-tile code is the single-volume frame's (march_fused, blend_rows,
-// blend_fused), so every pixel equals its volume's own frame bit for bit.
+// march_fused), so every pixel equals its volume's own frame bit for bit.
 #include "mboit_grid.cuh"
 
 namespace mb {
 namespace {
 
 template <class Cfg, bool kCache>
-__global__ void __launch_bounds__(256, Cfg::kVec ? 5 : 4) k_pass1_multi(const __grid_constant__ GridTable gt, const float4* __restrict__ tf,
+__global__ void __launch_bounds__(256, 4) k_pass1_multi(const __grid_constant__ GridTable gt, const float4* __restrict__ tf,
                                                         const __grid_constant__ ViewTable vt, char* __restrict__ moments,
                                                         Counters* __restrict__ ctr, const TileCache cache) {
     __shared__ float2 s_sig[256];
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) k_pass2_multi(const __grid_constant__ Gri
             const int kmin = __reduce_min_sync(0xffffffffu, k0), kmax = __reduce_max_sync(0xffffffffu, k1);
             blend_rows<false>(g, cache.vals + tb * 32, kmin, kmax, k0, k1, win, body);
         } else {
-            blend_fused<Cfg, false>(g, nullptr, win, o, d, k0, k1, body);
+            march_fused<Cfg, false>(g, nullptr, win, o, d, k0, k1, body);
         }
         if (valid) {
             const bool raw = (g.flags & kFlagRawSum) != 0;

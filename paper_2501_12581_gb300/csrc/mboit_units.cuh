@@ -859,6 +859,18 @@ __device__ __forceinline__ void march_amr_bricks(const AmrD& a, const float o_in
         else if (any)
             body(t, x);
     };
+    auto take2 = [&](float2 x, float ta, float tb, int j) {
+        if constexpr (kRows) {
+            store.put(x.x);
+            store.put(x.y);
+            body.add2(x.x, x.y, true, true, rows.z[j], rows.z[j + 1]);
+        } else if constexpr (HasPair<Body>::value) {
+            if (any) body.pair(make_float2(body.depth(ta), body.depth(tb)), x.x, x.y, true, true, __activemask());
+        } else {
+            take(x.x, ta, j);
+            take(x.y, tb, j + 1);
+        }
+    };
     store.seek(kmin);   // lanes without samples store too, into their slots of rows that other lanes hold
     for (int kw = kmin; kw <= kmax; kw += kDepthRows) {
         if constexpr (kRows) rows.fill(kw, g.step, body.wa, body.wb);
@@ -870,9 +882,7 @@ __device__ __forceinline__ void march_amr_bricks(const AmrD& a, const float o_in
                 float2 p[3];
                 uint32_t w[2];
                 brick_words(a, o, d, make_float2(t, tb), p, w);
-                const float2 x = brick_values(a, p, w);
-                take(x.x, t, j);
-                take(x.y, tb, j + 1);
+                take2(brick_values(a, p, w), t, tb, j);
                 t = tb + g.step;
             }
         } else {
@@ -1160,6 +1170,9 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 2>::value : 2) k_p
                                                                                k1, buf, body);
         } else if constexpr (kCache && (MS == 3 || MS == 4)) {
             march_uncached<kSel>(a, sel, o, d, k0, k1, body);
+        } else if (std::is_same<V, AmrD>::value && __all_sync(0xffffffffu, k0 > k1 || body.pairs())) {
+            PairBlend<typename Bodies<MS>::Blend> pb{body};
+            march_unit<kSel>(a, sel, o, d, k0, k1, pb);
         } else {
             march_unit<kSel>(a, sel, o, d, k0, k1, body);
         }
