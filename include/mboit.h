@@ -426,7 +426,10 @@ MBOIT_API mboit_status mboit_render_sortlast(mboit_volume v, const mboit_view* v
  * 11 x 8, whose dense layout spreads shared-memory banks; both also need the
  * driver's tensor-map encoder; otherwise MBOIT_ERR_INVALID_ARG and nothing
  * changes.  Every configuration gives the same bits.  Takes effect for the
- * next call; captured frame graphs are re-recorded. */
+ * next call; captured frame graphs are re-recorded.  Until this or
+ * mboit_autotune is called, each render takes the configuration its views
+ * suggest: 6 / 3 (where they can run) when neighbouring rays lie close
+ * together in the grid, else 0; mboit_stats tells which. */
 MBOIT_API mboit_status mboit_set_tuning(mboit_volume v, int32_t pass1, int32_t pass2);
 
 /* Number of kernel launches of mboit_render_frame: 2 (pass 1, then pass 2

@@ -92,6 +92,8 @@ struct mboit_volume_s {
     long long* d_tile_base = nullptr;
     unsigned long long* d_rows = nullptr;
     size_t cap_tcvals = 0, cap_tile_base = 0;
+    std::vector<char> multi_key;               // the last multi-volume frame's views and domains,
+    unsigned long long multi_rows = 0;         //   and the cache rows they take
     int32_t* d_bin_start = nullptr;
     int32_t* d_bin_tets = nullptr;
     float* d_tvals = nullptr;   // staging of host vertex values (mboit_render_frame_host)
@@ -114,6 +116,7 @@ struct mboit_volume_s {
     bool frame_timed = false;
     std::vector<GraphEntry> graphs;
     int32_t tune1 = 0, tune2 = 0;
+    bool tuned = false;         // set by mboit_set_tuning or the autotuner; else the views choose (auto_tune)
     CUtensorMap field_map[2];   // grids: the field's tensor maps for TMA windows (configurations 5 and 6)
     bool has_field_map = false;
     int32_t packet = MBOIT_PACKET_8X4;
@@ -140,6 +143,7 @@ struct mboit_volume_s {
 namespace {
 
 constexpr double kOneMarchVolume = 0.5;   // see one_march
+constexpr double kDenseRays = 0.75;       // see auto_tune
 constexpr double kTrigZone = 0.1;  // wrapping zone: phi = z (1 - zeta) pi
 
 // Angle map and the coefficients of s^m in (s + i)^k (s - i)^(n-k).
@@ -353,6 +357,7 @@ mboit_status build_views(const mboit_view* views, int32_t n_views, mb::ViewTable
         const int tw = 1 << S.tw_log2, th = 32 >> S.tw_log2;
         S.ntx = (V.width + tw - 1) / tw;
         const int64_t nty = (V.height + th - 1) / th;
+        S.nty = (int32_t)nty;
         S.tile_base = (int32_t)tiles;
         tiles += (int64_t)S.ntx * nty;
         S.plane = (int32_t)((((int64_t)V.width * V.height) + 3) / 4 * 4);
@@ -635,6 +640,35 @@ bool config_usable(mboit_volume v, int cfg) {
     return mb::stage_config_eligible(v->grid, cfg) && ((cfg != 5 && cfg != 6) || v->has_field_map);
 }
 
+// Window configurations of a grid nobody has tuned: 6 (of the sets that have
+// it, else 3) for pass 1 and 3 for pass 2 where neighbouring rays lie within
+// kDenseRays cells of each other at the domain's middle, so that a warp's window
+// spans many lattice steps; else 0, whose small windows fall back to direct
+// loads soonest.  Measured, one-launch frames in configurations 0 / 6: 256^3
+// at 1024^2 (0.42 cells) 1115 / 965 us, 256 x 96 x 320 at 900 x 700 434 / 330,
+// 64^3 at 256^2 (0.43) 95 / 92; 256^3 at 256^2 (1.7) 605 / 755.
+void auto_tune(mboit_volume v, const mb::ViewTable& vt) {
+    if (v->tuned || v->kind != MBOIT_GRID) return;
+    const mb::GridD& g = v->grid;
+    double spread = 0.0;
+    for (int i = 0; i < vt.n; ++i) {
+        const mb::ViewD& V = vt.s[i].v;
+        double dist = 0.0, u = 0.0, w = 0.0;
+        const double c[3] = {0.5 * g.hx - V.eye[0], 0.5 * g.hy - V.eye[1], 0.5 * g.hz - V.eye[2]};
+        for (int k = 0; k < 3; ++k) {
+            dist += c[k] * c[k];
+            u += (double)V.u[k] * V.u[k];
+            w += (double)V.v[k] * V.v[k];
+        }
+        const double far = V.projection == MBOIT_PERSPECTIVE ? 2.0 * std::sqrt(dist) : 1.0;
+        spread = std::max(spread, far * std::max(std::sqrt(u) * std::fabs(V.scale_u) / V.width,
+                                                 std::sqrt(w) * std::fabs(V.scale_v) / V.height));
+    }
+    const bool dense = spread <= kDenseRays;
+    v->tune1 = !dense ? 0 : config_usable(v, 6) ? 6 : config_usable(v, 3) ? 3 : 0;
+    v->tune2 = dense && config_usable(v, 3) ? 3 : 0;
+}
+
 // Checks the octree's or mesh's index tables on stream s before passes that
 // read them (grids have none).
 cudaError_t check_tables(mboit_volume v, cudaStream_t s) {
@@ -645,7 +679,7 @@ cudaError_t check_tables(mboit_volume v, cudaStream_t s) {
 
 cudaError_t pass1_batched(mboit_volume v, const uint8_t* mask, const mb::ViewTable& vt, void* moments, cudaStream_t s,
                           mb::TileCache tc = mb::TileCache{}) {
-    const cudaError_t e = check_tables(v, s);
+    const cudaError_t e = tc.cleared ? cudaSuccess : check_tables(v, s);
     if (e != cudaSuccess) return e;
     if (v->kind == MBOIT_AMR) return mb::launch_pass1_amr(v->amr, v->d_tf, mask, vt, moments, v->d_ctr, s, tc);
     if (v->kind == MBOIT_TET) return mb::launch_pass1_tet(v->tet, v->d_tf, mask, vt, moments, v->d_ctr, s, tc);
@@ -655,7 +689,7 @@ cudaError_t pass1_batched(mboit_volume v, const uint8_t* mask, const mb::ViewTab
 
 cudaError_t pass2_batched(mboit_volume v, const uint8_t* mask, const mb::ViewTable& vt, const void* moments,
                           float* color, int32_t mode, cudaStream_t s, mb::TileCache tc = mb::TileCache{}) {
-    const cudaError_t e = check_tables(v, s);
+    const cudaError_t e = tc.cleared ? cudaSuccess : check_tables(v, s);
     if (e != cudaSuccess) return e;
     if (v->kind == MBOIT_AMR)
         return mb::launch_pass2_amr(v->amr, v->d_tf, mask, vt, moments, color, mode, v->d_ctr, s, tc);
@@ -667,7 +701,7 @@ cudaError_t pass2_batched(mboit_volume v, const uint8_t* mask, const mb::ViewTab
 // The one-launch frame of the volume's kind (four power moments).
 cudaError_t frame_batched(mboit_volume v, const uint8_t* mask, const mb::ViewTable& vt, void* moments, float* color,
                           cudaStream_t s, int cfg, mb::TileCache tc) {
-    const cudaError_t e = check_tables(v, s);
+    const cudaError_t e = tc.cleared ? cudaSuccess : check_tables(v, s);
     if (e != cudaSuccess) return e;
     if (v->kind == MBOIT_AMR)
         return mb::launch_frame_amr(v->amr, v->d_tf, mask, vt, moments, color, mb::kColorResolved, v->d_ctr, s, tc);
@@ -738,11 +772,13 @@ mboit_status make_tile_order(mboit_volume v, const mb::ViewTable& vt, int32_t** 
 mboit_status cache_buffers(mboit_volume v, unsigned long long rows, int32_t total_tiles, mb::TileCache& c) {
     c = mb::TileCache{};
     const size_t nvals = (size_t)rows * 32, ntiles = (size_t)std::max(total_tiles, 1);
-    size_t free_b = 0, total_b = 0;
-    MB_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const size_t grow = (nvals > v->cap_tcvals ? nvals * sizeof(float) : 0) +
                         (ntiles > v->cap_tile_base ? ntiles * sizeof(long long) : 0);
-    if (grow + (size_t(1) << 30) > free_b) return MBOIT_OK;
+    if (grow > 0) {
+        size_t free_b = 0, total_b = 0;
+        MB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        if (grow + (size_t(1) << 30) > free_b) return MBOIT_OK;
+    }
     float* b1 = v->d_tcvals;
     long long* b2 = v->d_tile_base;
     MB_CUDA(ensure_capacity(v->d_tcvals, v->cap_tcvals, std::max<size_t>(nvals, 32)));
@@ -1278,6 +1314,7 @@ mboit_status mboit_render_moments(mboit_volume v, const mboit_view* views, int32
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = claim_stream(v, s)) != MBOIT_OK) return st;
     MB_CUDA(cudaMemsetAsync(&v->d_ctr->samples[0], 0, sizeof(unsigned long long), s));
+    auto_tune(v, vt);
     if (mode == MBOIT_MOMENTS_REDUCED) {
         MB_CUDA(pass1_batched(v, mask, vt, moments, s));
     } else {
@@ -1325,8 +1362,8 @@ mboit_status mboit_reconstruct_blend(mboit_volume v, const mboit_view* views, in
     if ((st = select_pieces(v, pieces, n_pieces, list, &mask)) != MBOIT_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = claim_stream(v, s)) != MBOIT_OK) return st;
-    MB_CUDA(cudaMemsetAsync(&v->d_ctr->samples[1], 0, 2 * sizeof(unsigned long long), s));
-    MB_CUDA(cudaMemsetAsync(&v->d_ctr->fp64_pixels, 0, sizeof(unsigned long long), s));
+    MB_CUDA(cudaMemsetAsync(&v->d_ctr->samples[1], 0, 3 * sizeof(unsigned long long), s));   // and singular, fp64_pixels
+    auto_tune(v, vt);
     if (mode == MBOIT_COLOR_PER_PIECE) {
         const int32_t slots = (int32_t)list.size();
         MB_CUDA(check_tables(v, s));
@@ -1408,6 +1445,7 @@ mboit_status mboit_render_frame(mboit_volume v, const mboit_view* views, int32_t
     const uint8_t* mask = nullptr;
     if ((st = select_pieces(v, nullptr, 0, list, &mask)) != MBOIT_OK) return st;
     if ((st = claim_stream(v, static_cast<cudaStream_t>(stream))) != MBOIT_OK) return st;
+    auto_tune(v, vt);
     // graph key: the view table and the output pointers
     std::vector<char> key(sizeof vt + 2 * sizeof(void*));
     std::memcpy(key.data(), &vt, sizeof vt);
@@ -1424,8 +1462,9 @@ mboit_status mboit_render_frame(mboit_volume v, const mboit_view* views, int32_t
         vt.order = d_order;
         cudaStream_t cs = v->cap_stream;
         MB_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = cudaMemsetAsync(&v->d_ctr->samples[0], 0, 3 * sizeof(unsigned long long), cs);
-        if (e == cudaSuccess) e = cudaMemsetAsync(&v->d_ctr->fp64_pixels, 0, sizeof(unsigned long long), cs);
+        cudaError_t e = mb::clear_frame_counters(v->d_ctr, cs);
+        if (e == cudaSuccess) e = check_tables(v, cs);
+        tc.cleared = 1;
         // external record nodes: the events are recorded each time the graph runs
         if (e == cudaSuccess) e = cudaEventRecordWithFlags(v->frame_ev[0], cs, cudaEventRecordExternal);
         if (v->frame_launches == 1) {
@@ -1519,28 +1558,40 @@ mboit_status mboit_render_frame_multi(const mboit_volume* vols, int32_t n_vols, 
         }
     }
     for (int32_t i = 0; i < n_views; ++i) vt.s[i].vol = view_volume[i];
-    // the sample cache: rows of every volume's views, counted per volume
-    cudaStream_t cs = v0->cap_stream;
-    if (!v0->d_rows) MB_CUDA(cudaMalloc(&v0->d_rows, sizeof(unsigned long long)));
-    MB_CUDA(cudaMemsetAsync(v0->d_rows, 0, sizeof(unsigned long long), cs));
+    // the sample cache: rows of every volume's views, counted per volume; they
+    // depend on the views and the domains only, so a repeated call keeps the
+    // count (and waits for nothing)
+    std::vector<char> key(sizeof vt);
+    std::memcpy(key.data(), &vt, sizeof vt);
     for (int32_t i = 0; i < n_vols; ++i) {
-        std::vector<mboit_view> mine;
-        for (int32_t j = 0; j < n_views; ++j)
-            if (view_volume[j] == i) mine.push_back(views[j]);
-        if (mine.empty()) continue;
-        mb::ViewTable sub;
-        if ((st = build_views(mine.data(), (int32_t)mine.size(), sub, slab_bytes_per_px(MBOIT_POWER4), v0->packet)) !=
-            MBOIT_OK)
-            return st;
-        MB_CUDA(mb::launch_tile_rows(gt.g[i], sub, v0->d_rows, cs));
+        const float dom[4] = {gt.g[i].hx, gt.g[i].hy, gt.g[i].hz, gt.g[i].step};
+        key.insert(key.end(), (const char*)dom, (const char*)dom + sizeof dom);
     }
-    unsigned long long rows = 0;
-    MB_CUDA(cudaMemcpyAsync(&rows, v0->d_rows, sizeof rows, cudaMemcpyDeviceToHost, cs));
-    MB_CUDA(cudaStreamSynchronize(cs));
+    unsigned long long rows = v0->multi_rows;
+    if (key != v0->multi_key) {
+        cudaStream_t cs = v0->cap_stream;
+        if (!v0->d_rows) MB_CUDA(cudaMalloc(&v0->d_rows, sizeof(unsigned long long)));
+        MB_CUDA(cudaMemsetAsync(v0->d_rows, 0, sizeof(unsigned long long), cs));
+        for (int32_t i = 0; i < n_vols; ++i) {
+            std::vector<mboit_view> mine;
+            for (int32_t j = 0; j < n_views; ++j)
+                if (view_volume[j] == i) mine.push_back(views[j]);
+            if (mine.empty()) continue;
+            mb::ViewTable sub;
+            if ((st = build_views(mine.data(), (int32_t)mine.size(), sub, slab_bytes_per_px(MBOIT_POWER4), v0->packet)) !=
+                MBOIT_OK)
+                return st;
+            MB_CUDA(mb::launch_tile_rows(gt.g[i], sub, v0->d_rows, cs));
+        }
+        MB_CUDA(cudaMemcpyAsync(&rows, v0->d_rows, sizeof rows, cudaMemcpyDeviceToHost, cs));
+        MB_CUDA(cudaStreamSynchronize(cs));
+        v0->multi_key.swap(key);
+        v0->multi_rows = rows;
+    }
     mb::TileCache tc;
     if ((st = cache_buffers(v0, rows, vt.total_tiles, tc)) != MBOIT_OK) return st;
-    MB_CUDA(cudaMemsetAsync(&v0->d_ctr->samples[0], 0, 3 * sizeof(unsigned long long), s));
-    MB_CUDA(cudaMemsetAsync(&v0->d_ctr->fp64_pixels, 0, sizeof(unsigned long long), s));
+    MB_CUDA(mb::clear_frame_counters(v0->d_ctr, s));
+    tc.cleared = 1;
     if (amr) {
         // every octree's index tables checked on this stream first (its error word)
         for (int32_t i = 0; i < n_vols; ++i) MB_CUDA(check_tables(vols[i], s));
@@ -1740,6 +1791,7 @@ mboit_status mboit_set_tuning(mboit_volume v, int32_t pass1, int32_t pass2) {
     std::lock_guard<std::mutex> lk(v->mu);
     v->tune1 = pass1;
     v->tune2 = pass2;
+    v->tuned = true;
     drop_graphs(v);
     return MBOIT_OK;
 }
@@ -1836,6 +1888,7 @@ mboit_status mboit_autotune(mboit_volume v, const mboit_view* views, int32_t n_v
         const auto it = g_tuned.find(key);
         if (it != g_tuned.end()) {
             const Tuned& t = it->second;
+            v->tuned = true;
             v->tune1 = t.tune1;
             v->tune2 = t.tune2;
             v->packet = t.packet;
@@ -1989,6 +2042,7 @@ mboit_status mboit_autotune(mboit_volume v, const mboit_view* views, int32_t n_v
     if (ce != cudaSuccess) return fail(MBOIT_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(ce));
     v->frame_launches = launches;
     v->tile_order = order;
+    v->tuned = true;
     v->tune1 = best[0];
     v->tune2 = best[1];
     v->packet = best[2];

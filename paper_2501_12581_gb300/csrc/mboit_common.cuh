@@ -686,12 +686,30 @@ __device__ __forceinline__ void count_frames(Counters* ctr, const Body& body, bo
 }
 
 // Pops the next 8x4 ray tile of the work queue; returns false when empty.
+// Without an order table (kMiddle) a view's rows of tiles come from the middle
+// outward: rays through the middle of a view are the long ones, so the queue
+// ends on short tiles and the last warps run alone for less time (two 512^2
+// views of 2,367 leaves: 670 -> 642 us; half of a 256^3 grid's pieces, 1024 x
+// 768: 1069 -> 1044).  Not when every warp takes one or two tiles: then it puts
+// the long ones on the same SMs (64^3 at 256^2: 95 -> 104 us); nor in the
+// one-launch grid frame, whose long tiles keep both passes' units busy
+// (301 x 227 x 181 at 1000 x 723: 587 -> 592); nor with the other moment sets
+// (half to one percent slower).
+template <bool kMiddle = true>
 __device__ __forceinline__ bool next_tile(const ViewTable& vt, int32_t* head, int& vi, int& px, int& py, int& tile) {
     const int lane = threadIdx.x & 31;
     tile = 0;
     if (lane == 0) {
         tile = atomicAdd(head, 1);
-        if (vt.order && tile < vt.total_tiles) tile = __ldg(vt.order + tile);
+        if (tile < vt.total_tiles) {
+            if (vt.order) {
+                tile = __ldg(vt.order + tile);
+            } else if (kMiddle && vt.total_tiles > 2 * (int)(gridDim.x * kFusedWarps)) {
+                const ViewSlot& S = vt.s[find_view(vt, tile)];
+                const int lt = tile - S.tile_base, k = lt / S.ntx, mid = S.nty >> 1;
+                tile += ((k & 1 ? mid - ((k + 1) >> 1) : mid + (k >> 1)) - k) * S.ntx;
+            }
+        }
     }
     tile = __shfl_sync(0xffffffffu, tile, 0);
     if (tile >= vt.total_tiles) return false;

@@ -67,8 +67,7 @@ cudaError_t launch_pass1_fused(const GridD& g, const float4* tf, const uint8_t* 
                                const CUtensorMap* tmap) {
     if (!stage_config_eligible(g, cfg)) cfg = 0;
     if ((cfg == 5 || cfg == 6) && !tmap) cfg = 3;   // no tensor map: a window by plain loads
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && cache.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = brick_sel != nullptr;
     const void* fn = cache.vals ? pass1_fn<true>(cfg, sel, g.trig.sel) : pass1_fn(cfg, sel, g.trig.sel);
@@ -115,7 +114,7 @@ cudaError_t launch_pass2_fused(const GridD& g, const float4* tf, const uint8_t* 
                                const void* moments, float* color, int32_t mode, Counters* ctr, cudaStream_t s,
                                int cfg, TileCache cache) {
     if (!stage_config_eligible(g, cfg)) cfg = 0;
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+    cudaError_t e = clear_pass2_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = brick_sel != nullptr;
     const void* fn = cache.vals ? pass2_fn<true>(cfg, sel, g.trig.sel) : pass2_fn(cfg, sel, g.trig.sel);

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(256, 4) k_pass1_fused(const __grid_constant__ 
     float* win = s_win[threadIdx.x >> 5];
     TmaWin tw{&tmap, s_bar + (Cfg::kTma ? threadIdx.x >> 5 : 0), 0u, &ctr->error, (g.flags & kFlagDebugNoCopy) != 0};
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[0], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[0], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         float o[3], d[3];
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(256) k_pass2_fused(const __grid_constant__ Gri
     float* win = s_win[threadIdx.x >> 5];
     const bool raw = (g.flags & 1u) != 0;
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[1], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[1], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         const int pix = valid ? py * S.v.width + px : 0;
@@ -474,6 +474,8 @@ __global__ void __launch_bounds__(256) k_pass2_fused(const __grid_constant__ Gri
 
 template <int MS, bool kC>
 const void* pass1_fn_ms(int cfg, bool sel) {
+    if constexpr (MS == 0)
+        if (sel && (cfg == 3 || cfg == 5 || cfg == 6)) return (const void*)k_pass1_fused<true, Stage3, MS, kC>;
     if (sel) return (const void*)k_pass1_fused<true, Stage0, MS, kC>;
     if constexpr (MS != 0) {
         // other moment sets: configurations 0 and 3 only
@@ -494,6 +496,8 @@ const void* pass1_fn_ms(int cfg, bool sel) {
 
 template <int MS, bool kC>
 const void* pass2_fn_ms(int cfg, bool sel) {
+    if constexpr (MS == 0)
+        if (sel && (cfg == 3 || cfg == 5 || cfg == 6)) return (const void*)k_pass2_fused<true, Stage3, MS, kC>;
     if (sel) return (const void*)k_pass2_fused<true, Stage0, MS, kC>;
     if constexpr (MS != 0) {
         // other moment sets: configurations 0 and 3 only

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) k_frame_fused(const __grid_constant__ Gri
     TmaWin tw{&tmap, s_bar + (Cfg::kTma ? threadIdx.x >> 5 : 0), 0u, &ctr->error, (g.flags & kFlagDebugNoCopy) != 0};
     const bool raw = (g.flags & 1u) != 0;
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[0], vi, px, py, tile)) {
+    while (next_tile<false>(vt, &ctr->tile_next[0], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         const int pix = valid ? py * S.v.width + px : 0;
@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(256) k_frame_fused(const __grid_constant__ Gri
 }
 
 const void* frame_fn(int cfg, bool sel) {
+    if (sel && (cfg == 3 || cfg == 5 || cfg == 6)) return (const void*)k_frame_fused<true, Stage3>;
     if (sel) return (const void*)k_frame_fused<true, Stage0>;
     switch (cfg) {
         case 1: return (const void*)k_frame_fused<false, Stage1>;
@@ -124,8 +125,7 @@ cudaError_t launch_frame_fused(const GridD& g, const float4* tf, const uint8_t* 
                                TileCache cache, const CUtensorMap* tmap) {
     if (!stage_config_eligible(g, cfg)) cfg = 0;
     if ((cfg == 5 || cfg == 6) && !tmap) cfg = 3;
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = frame_fn(cfg, brick_sel != nullptr);
     char* m = static_cast<char*>(moments);

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(256, 4) k_pass1_multi(const __grid_constant__ 
     __syncthreads();
     float* win = s_win[threadIdx.x >> 5];
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[0], vi, px, py, tile)) {
+    while (next_tile<false>(vt, &ctr->tile_next[0], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const GridD& g = gt.g[S.vol];
         const bool valid = px < S.v.width && py < S.v.height;
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) k_pass2_multi(const __grid_constant__ Gri
     __syncthreads();
     float* win = s_win[threadIdx.x >> 5];
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[1], vi, px, py, tile)) {
+    while (next_tile<false>(vt, &ctr->tile_next[1], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const GridD& g = gt.g[S.vol];
         const bool valid = px < S.v.width && py < S.v.height;
@@ -115,8 +115,7 @@ cudaError_t prepare_multi_kernels() {
 
 cudaError_t launch_pass1_multi(const GridTable& gt, const float4* tf, const ViewTable& vt, void* moments,
                                Counters* ctr, cudaStream_t s, bool vec, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && cache.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = cache.vals ? pass1_multi_fn<true>(vec) : pass1_multi_fn<false>(vec);
     char* m = static_cast<char*>(moments);
@@ -126,7 +125,7 @@ cudaError_t launch_pass1_multi(const GridTable& gt, const float4* tf, const View
 
 cudaError_t launch_pass2_multi(const GridTable& gt, const float4* tf, const ViewTable& vt, const void* moments,
                                float* color, Counters* ctr, cudaStream_t s, bool vec, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+    cudaError_t e = clear_pass2_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = cache.vals ? pass2_multi_fn<true>(vec) : pass2_multi_fn<false>(vec);
     const char* m = static_cast<const char*>(moments);

@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda.h>   // CUtensorMap (the type only; the library calls the driver through the runtime's entry point)
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "mboit_device.cuh"
@@ -21,7 +22,7 @@ struct ViewSlot {
     int32_t plane;          // pixels per moment plane (w*h rounded up to 4)
     int32_t tw_log2;        // a warp's ray tile (packet) is 2^tw_log2 x 2^(5 - tw_log2) pixels: 8 x 4 or 4 x 8
     int32_t vol;            // multi-volume frames: the view's volume in the GridTable (else 0)
-    int32_t pad;
+    int32_t nty;            // rows of tiles
 };
 
 // Pixel of lane `lane` in tile `lt` of a view (tiles row-major, ntx per row).
@@ -35,8 +36,8 @@ struct ViewTable {
     int32_t n;
     int32_t total_tiles;
     // dequeue order: the queue's i-th pop takes tile order[i] (a permutation of
-    // the tiles, longest first); NULL: tiles in order (views in turn, rows of
-    // tiles top to bottom)
+    // the tiles, longest first); NULL: views in turn, rows of tiles from the
+    // middle outward (next_tile)
     const int32_t* order;
     ViewSlot s[kMaxViews];
 };
@@ -51,16 +52,20 @@ constexpr int32_t kErrTmaTimeout = 0x10;  // a TMA window load did not complete 
 // Device counters owned by a volume.
 struct Counters {
     int32_t tile_next[4];            // work-queue heads, one per concurrent pass
-    int32_t error;                   // kErr* bits of the kernel-side checks that failed since the last read
-    int32_t pad;
+    unsigned long long cache_rows;   // rows of the frame's sample cache handed out so far
     unsigned long long samples[2];   // pass 1, pass 2
     unsigned long long singular;     // pixels on a 1-/2-atom branch
+    unsigned long long fp64_pixels;  // pixels whose reconstruction frame was set up in FP64
+    // a frame clears what stands above at once (clear_frame_counters)
+    int32_t error;                   // kErr* bits of the kernel-side checks that failed since the last read
+    int32_t pad;
     unsigned long long segments;     // sort-last segments of the last baseline frame
     int32_t max_segments;            // most segments on one pixel
     int32_t pad2;
-    unsigned long long cache_rows;   // rows of the frame's sample cache handed out so far
-    unsigned long long fp64_pixels;  // pixels whose reconstruction frame was set up in FP64
 };
+inline cudaError_t clear_frame_counters(Counters* ctr, cudaStream_t s) {
+    return cudaMemsetAsync(ctr, 0, offsetof(Counters, error), s);
+}
 
 struct PieceBox {
     float lo[3], hi[3];              // voxel-space box covering the piece's bricks
@@ -131,7 +136,23 @@ struct TileCache {
     float* vals;
     long long* tile_base;
     long long rows_cap;
+    // 1: this frame's counters are cleared and its tables checked already (its
+    // launches then do neither: each such node costs a small frame 1 to 3 us)
+    int32_t cleared;
+    int32_t pad;
 };
+
+// The queue head and the cache's row counter of a pass, unless the frame has
+// cleared its counters.
+inline cudaError_t clear_pass1_counters(Counters* ctr, const TileCache& c, cudaStream_t s) {
+    if (c.cleared) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
+    if (e == cudaSuccess && c.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    return e;
+}
+inline cudaError_t clear_pass2_counters(Counters* ctr, const TileCache& c, cudaStream_t s) {
+    return c.cleared ? cudaSuccess : cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+}
 
 // Number of shared-memory window configurations of the fused passes (the
 // autotuner's choices).  Configurations 2-6 use 16-byte loads and need

@@ -117,8 +117,7 @@ cudaError_t prepare_multi_amr_kernels() {
 
 cudaError_t launch_pass1_multi_amr(const AmrTable& at, const float4* tf, const ViewTable& vt, void* moments,
                                    Counters* ctr, cudaStream_t s, bool sel, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && cache.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = cache.vals ? pass1_fn<true>(sel) : pass1_fn<false>(sel);
     char* m = static_cast<char*>(moments);
@@ -128,7 +127,7 @@ cudaError_t launch_pass1_multi_amr(const AmrTable& at, const float4* tf, const V
 
 cudaError_t launch_pass2_multi_amr(const AmrTable& at, const float4* tf, const ViewTable& vt, const void* moments,
                                    float* color, Counters* ctr, cudaStream_t s, bool sel, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+    cudaError_t e = clear_pass2_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = cache.vals ? pass2_fn<true>(sel) : pass2_fn<false>(sel);
     const char* m = static_cast<const char*>(moments);

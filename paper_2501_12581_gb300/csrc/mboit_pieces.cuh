@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256, MS == 0 ? PieceMinBlocks<V>::value : 2)
     }
     __syncthreads();
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[0], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[0], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         float o[3], d[3];
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(256, MS == 0 ? PieceMinBlocks<V>::value : 2)
     }
     __syncthreads();
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[1], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[1], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         const int pix = valid ? py * S.v.width + px : 0;

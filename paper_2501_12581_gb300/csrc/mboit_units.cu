@@ -176,8 +176,7 @@ cudaError_t launch_sortlast_march(bool fill, const GridD& g, const float4* tf, c
 
 cudaError_t launch_pass1_amr(const AmrD& a, const float4* tf, const uint8_t* unit_sel, const ViewTable& vt,
                              void* moments, Counters* ctr, cudaStream_t s, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && cache.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = unit_sel != nullptr || !a.complete;   // octrees with holes take the checked kernels
     const void* fn = cache.vals ? unit1_fn<AmrD, true>(sel, a.g.trig.sel) : unit1_fn<AmrD>(sel, a.g.trig.sel);
@@ -189,7 +188,7 @@ cudaError_t launch_pass1_amr(const AmrD& a, const float4* tf, const uint8_t* uni
 cudaError_t launch_pass2_amr(const AmrD& a, const float4* tf, const uint8_t* unit_sel, const ViewTable& vt,
                              const void* moments, float* color, int32_t mode, Counters* ctr, cudaStream_t s,
                              TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+    cudaError_t e = clear_pass2_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = unit_sel != nullptr || !a.complete;
     const void* fn = cache.vals ? unit2_fn<AmrD, true>(sel, a.g.trig.sel) : unit2_fn<AmrD>(sel, a.g.trig.sel);
@@ -240,8 +239,7 @@ TetT<kN> as_tet(const TetD& m) {
 template <class V>
 cudaError_t launch_unit1(const V& vol, const float4* tf, const uint8_t* unit_sel, const ViewTable& vt, void* moments,
                          Counters* ctr, cudaStream_t s, TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && cache.vals) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = unit_sel != nullptr;
     const void* fn = cache.vals ? unit1_fn<V, true>(sel, vol.g.trig.sel) : unit1_fn<V>(sel, vol.g.trig.sel);
@@ -254,7 +252,7 @@ template <class V>
 cudaError_t launch_unit2(const V& vol, const float4* tf, const uint8_t* unit_sel, const ViewTable& vt,
                          const void* moments, float* color, int32_t mode, Counters* ctr, cudaStream_t s,
                          TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[1], 0, sizeof(int32_t), s);
+    cudaError_t e = clear_pass2_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const bool sel = unit_sel != nullptr;
     const void* fn = cache.vals ? unit2_fn<V, true>(sel, vol.g.trig.sel) : unit2_fn<V>(sel, vol.g.trig.sel);

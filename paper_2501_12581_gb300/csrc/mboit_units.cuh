@@ -1102,7 +1102,7 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 1>::value : 2) k_p
     const GridD& g = a.g;
     float4* zrows = s_z[threadIdx.x >> 5];
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[0], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[0], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         float o[3], d[3];
@@ -1144,7 +1144,7 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 2>::value : 2) k_p
     const GridD& g = a.g;
     const bool raw = (g.flags & 1u) != 0;
     int vi, px, py, tile;
-    while (next_tile(vt, &ctr->tile_next[1], vi, px, py, tile)) {
+    while (next_tile<MS == 0>(vt, &ctr->tile_next[1], vi, px, py, tile)) {
         const ViewSlot& S = vt.s[vi];
         const bool valid = px < S.v.width && py < S.v.height;
         const int pix = valid ? py * S.v.width + px : 0;

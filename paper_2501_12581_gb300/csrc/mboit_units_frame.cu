@@ -113,8 +113,7 @@ template <class V>
 cudaError_t launch_frame_unit(const V& vol, const float4* tf, const uint8_t* unit_sel, const ViewTable& vt,
                               void* moments, float* color, int32_t mode, Counters* ctr, cudaStream_t s,
                               TileCache cache) {
-    cudaError_t e = cudaMemsetAsync(&ctr->tile_next[0], 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&ctr->cache_rows, 0, sizeof(unsigned long long), s);
+    cudaError_t e = clear_pass1_counters(ctr, cache, s);
     if (e != cudaSuccess) return e;
     const void* fn = frame_unit_fn<V>(unit_sel != nullptr || !complete_units(vol));
     char* mo = static_cast<char*>(moments);
