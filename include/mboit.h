@@ -286,7 +286,9 @@ MBOIT_API mboit_status mboit_destroy_volume(mboit_volume v);
 MBOIT_API mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int32_t ids_on_device,
                              int32_t* piece_id_out);
 
-/* Pass 1 (Sec. 4.1, Alg. 2).  views: HOST array of n_views views.  pieces:
+/* Pass 1 (Sec. 4.1, Alg. 2).  PER_PIECE images of many pieces come from one
+ * march per ray, of few from one march per piece; the same bits.  views: HOST
+ * array of n_views views.  pieces:
  * HOST array of n_pieces selected piece ids, or NULL = all pieces (then
  * n_pieces is ignored).  moments: DEVICE buffer of n_views * S bytes
  * (REDUCED) or n_views * n_pieces * S bytes (PER_PIECE), S =
@@ -348,8 +350,8 @@ MBOIT_API mboit_status mboit_render_frame(mboit_volume v, const mboit_view* view
  * 1 <= n_vols <= 8, 1 <= n_views <= 16.  moments_scratch and rgba are laid
  * out as for mboit_render_frame over the n_views views; every image equals,
  * bit for bit, its volume's own mboit_render_frame.  Pass 1 stores the
- * sample cache of vols[0] (sized for all views; synchronises once per call
- * to size it) and pass 2 blends from it; grid windows take configuration 3
+ * sample cache of vols[0] (sized for all views; synchronises to size it when
+ * the views or the domains are not those of the last such call) and pass 2 blends from it; grid windows take configuration 3
  * when every field qualifies (dims[0] % 4, alignment), else 0; octrees have
  * their tables checked first, each into its own error word
  * (mboit_synchronize on that volume reports a failure; that volume's tiles
@@ -445,7 +447,7 @@ MBOIT_API mboit_status mboit_set_frame_launches(mboit_volume v, int32_t launches
 
 /* Dequeue order of the ray tiles in mboit_render_frame (the batching
  * pattern's cost-ordered work items): 0 = tile order (views in turn, rows
- * of tiles top to bottom), 1 = longest first: when a frame graph is
+ * of tiles top to bottom or from a view's middle outward), 1 = longest first: when a frame graph is
  * recorded, one small kernel counts each ray tile's lattice rows (the rows
  * its warp walks in lockstep, the tile's cost) and the tiles are sorted by
  * it, so the persistent kernels start the long tiles early and end on
