@@ -74,13 +74,12 @@ __device__ __forceinline__ bool field_sample(const GridD& g, const uint8_t* __re
 // replaces share a slower pipe.
 struct Split2 {
     float2 f;
-    int a, b;   // carry the bits of 2^23 (kSplitBias)
+    uint32_t a, b;   // carry the bits of 2^23 (kSplitBias)
 };
-constexpr int kSplitBias = 0x4b000000;
 __device__ __forceinline__ Split2 split2(float2 x) {
     const float2 m = __fadd2_rd(x, make_float2(8388608.0f, 8388608.0f));
     const float2 w = __fadd2_rn(m, make_float2(-8388608.0f, -8388608.0f));
-    return {__ffma2_rn(w, make_float2(-1.0f, -1.0f), x), __float_as_int(m.x), __float_as_int(m.y)};
+    return {__ffma2_rn(w, make_float2(-1.0f, -1.0f), x), __float_as_uint(m.x), __float_as_uint(m.y)};
 }
 
 // Transfer-function table coordinate of sample value v (O5): the value
@@ -262,7 +261,7 @@ __device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float
                                            bool oka, bool okb, bool live, bool thin, unsigned act,
                                            const T& transmittances) {
     const Split2 x = split2(make_float2(oka ? xa : 0.0f, okb ? xb : 0.0f));
-    const int ia = x.a - kSplitBias, ib = x.b - kSplitBias;
+    const uint32_t ia = x.a - kSplitBias, ib = x.b - kSplitBias;
     const float fa = x.f.x, fb = x.f.y;
     const float4 ea = s_tf[2 * ia], da = s_tf[2 * ia + 1], eb = s_tf[2 * ib], db = s_tf[2 * ib + 1];
     // the table lerps as pairs: (r, g) and (b, absorbance) of each point

@@ -136,6 +136,17 @@ MB_HD float fclamp(float x, float lo, float hi) { return fmin_(fmax_(x, lo), hi)
 
 constexpr float kLog2e = 1.4426950408889634f;
 
+// The float 2^23 as bits.  A whole number n in [0, 2^23) added to 2^23 carries
+// these bits plus n, so a table or cell index computed from such sums is right
+// modulo 2^32 once the same combination of kSplitBias is taken off.  Unsigned:
+// the sums leave 32 bits, which int must not.
+constexpr uint32_t kSplitBias = 0x4b000000u;
+// Combination of three indices (or of one bias three times) in a window with
+// `pitch` floats per row and `plane` per plane, modulo 2^32.
+MB_HD uint32_t window_offset(uint32_t x, uint32_t y, uint32_t z, uint32_t pitch, uint32_t plane) {
+    return z * plane + y * pitch + x;
+}
+
 // ---------------------------------------------------------------------------
 // views and volumes as the kernels see them
 

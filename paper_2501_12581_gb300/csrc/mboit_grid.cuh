@@ -258,7 +258,8 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
                 const float2 o0 = make_float2(o[0], o[0]), o1 = make_float2(o[1], o[1]), o2 = make_float2(o[2], o[2]);
                 const float2 d0 = make_float2(d[0], d[0]), d1 = make_float2(d[1], d[1]), d2 = make_float2(d[2], d[2]);
                 // the window's origin, and the bits that split2's whole parts carry (mod 2^32)
-                const int base = (LO[2] + kSplitBias) * Cfg::Plane + (LO[1] + kSplitBias) * Cfg::Pitch + LO[0] + kSplitBias;
+                const uint32_t base = window_offset((uint32_t)LO[0] + kSplitBias, (uint32_t)LO[1] + kSplitBias,
+                                                    (uint32_t)LO[2] + kSplitBias, Cfg::Pitch, Cfg::Plane);
                 for (; t0 + g.step <= tz; t0 += 2.0f * g.step) {
                     const float tb = t0 + g.step;
                     const float2 t2 = make_float2(t0, tb);
@@ -266,9 +267,10 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
                                  z = split2(__ffma2_rn(t2, d2, o2));
                     bool oka = true, okb = true;
                     if constexpr (kSel) {
-                        auto wanted = [&](int ix, int iy, int iz) {
-                            const int bx = (ix - kSplitBias) >> g.brick_log2, by = (iy - kSplitBias) >> g.brick_log2,
-                                      bz = (iz - kSplitBias) >> g.brick_log2;
+                        auto wanted = [&](uint32_t ix, uint32_t iy, uint32_t iz) {
+                            const int bx = (int)(ix - kSplitBias) >> g.brick_log2,
+                                      by = (int)(iy - kSplitBias) >> g.brick_log2,
+                                      bz = (int)(iz - kSplitBias) >> g.brick_log2;
                             return __ldg(sel + (bz * g.nby + by) * g.nbx + bx) != 0;
                         };
                         oka = wanted(x.a, y.a, z.a);
@@ -279,8 +281,8 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
                             continue;
                         }
                     }
-                    const float* ca = win + (z.a * Cfg::Plane + y.a * Cfg::Pitch + x.a - base);
-                    const float* cb = win + (z.b * Cfg::Plane + y.b * Cfg::Pitch + x.b - base);
+                    const float* ca = win + (int)(window_offset(x.a, y.a, z.a, Cfg::Pitch, Cfg::Plane) - base);
+                    const float* cb = win + (int)(window_offset(x.b, y.b, z.b, Cfg::Pitch, Cfg::Plane) - base);
                     auto at = [&](int k) { return make_float2(ca[k], cb[k]); };
                     auto lerp = [](float2 f, float2 v0, float2 v1) { return __ffma2_rn(f, fsub2(v1, v0), v0); };
                     const float2 lo = lerp(y.f, lerp(x.f, at(0), at(1)), lerp(x.f, at(Cfg::Pitch), at(Cfg::Pitch + 1)));
