@@ -253,12 +253,11 @@ struct DepthRows {
 // packed FP32x2 instruction with the scalar form's rounding, the colour sums
 // taken for a, then b, so that the result equals two one-point calls bit for
 // bit.  A point with ok = false adds nothing: its table coordinate is replaced
-// by 0 (no NaN enters) and its weight by 0, and fma(0, c, C) = C.  `live` false:
-// the pixel has no absorbance and its T may be NaN; nothing is added.  `thin`:
-// no absorbance reaches 1/4 (kFlagThin).  transmittances(): both T.
+// by 0 (no NaN enters) and its weight by 0, and fma(0, c, C) = C.  `thin`: no
+// absorbance reaches 1/4 (kFlagThin).  transmittances(): both T.
 template <class T>
 __device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float4& C, unsigned& n, float xa, float xb,
-                                           bool oka, bool okb, bool live, bool thin, unsigned act,
+                                           bool oka, bool okb, bool thin, unsigned act,
                                            const T& transmittances) {
     const Split2 x = split2(make_float2(oka ? xa : 0.0f, okb ? xb : 0.0f));
     const uint32_t ia = x.a - kSplitBias, ib = x.b - kSplitBias;
@@ -285,8 +284,8 @@ __device__ __forceinline__ void blend_pair(const float4* s_tf, float amax, float
         alpha = make_float2(a.x < 0.25f ? alpha.x : dir.x, a.y < 0.25f ? alpha.y : dir.y);
     }
     float2 wgt = __fmul2_rn(transmittances(), alpha);
-    wgt.x = oka && live ? wgt.x : 0.0f;
-    wgt.y = okb && live ? wgt.y : 0.0f;
+    wgt.x = oka ? wgt.x : 0.0f;
+    wgt.y = okb ? wgt.y : 0.0f;
     // colour sums as pairs: (r, g) and (b, alpha); C.w + w = fma(w, 1, C.w)
     float2 cxy = __ffma2_rn(make_float2(wgt.x, wgt.x), rga, make_float2(C.x, C.y));
     float2 czw = __ffma2_rn(make_float2(wgt.x, wgt.x), make_float2(bwa.x, 1.0f), make_float2(C.z, C.w));
@@ -326,12 +325,12 @@ struct BlendBody {
     __device__ __forceinline__ bool singular() const { return F.kind == kFrameOneAtom || F.kind == kFrameTwoAtoms; }
 
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
-    // Frames whose points pair_generic may take: generic ones, and pixels
-    // without absorbance, whose opacities are all 0 (T is finite there).
+    // Frames whose points pair may take: generic ones, and pixels without
+    // absorbance (an empty frame gives T = 1 in the same arithmetic).
     __device__ __forceinline__ bool pairs() const { return F.kind == kFrameGeneric || F.kind == kFrameEmpty; }
     // Two points of a generic frame: equal to two sample<true> calls bit for bit.
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, true, thin, act, [&]() {
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, thin, act, [&]() {
             const float2 ex = __fmul2_rn(make_float2(-F.m0_log2e, -F.m0_log2e), bound_generic2(F, z, w0, act));
             return make_float2(fexp2(ex.x), fexp2(ex.y));
         });
@@ -444,7 +443,10 @@ struct TrigMomentBody {
 };
 
 // T = e^(-b0 A) of two points, clamped to [0, 1] as the one-point bodies do.
-__device__ __forceinline__ float2 heavy_transmittance(float m0_log2e, float2 A) {
+// `live` false: the pixel has no absorbance, its frame is empty and A may be
+// NaN; nothing lies in front, A = 0 and T = 1.
+__device__ __forceinline__ float2 heavy_transmittance(float m0_log2e, float2 A, bool live) {
+    A = live ? A : make_float2(0.0f, 0.0f);
     const float2 ex = __fmul2_rn(make_float2(-m0_log2e, -m0_log2e), A);
     return make_float2(fclamp(fexp2(ex.x), 0.0f, 1.0f), fclamp(fexp2(ex.y), 0.0f, 1.0f));
 }
@@ -479,8 +481,8 @@ struct TrigBlendBody {
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
     __device__ __forceinline__ bool pairs() const { return !singular(); }
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.n != 0, thin, act,
-                   [&]() { return heavy_transmittance(F.m0_log2e, trig_fraction<N, float2>(F, *T, z, w0)); });
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, thin, act,
+                   [&]() { return heavy_transmittance(F.m0_log2e, trig_fraction<N, float2>(F, *T, z, w0), F.n != 0); });
     }
 };
 
@@ -568,8 +570,9 @@ struct PowerBlendBody {
     __device__ __forceinline__ float depth(float t) const { return warp_depth(t, wa, wb); }
     __device__ __forceinline__ bool pairs() const { return !singular(); }
     __device__ __forceinline__ void pair(float2 z, float xa, float xb, bool oka, bool okb, unsigned act) {
-        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, F.kind == kFrameGeneric, thin, act,
-                   [&]() { return heavy_transmittance(F.m0_log2e, power_fraction_generic<N, float2>(F, z, w0)); });
+        blend_pair(s_tf, amax, C, n, xa, xb, oka, okb, thin, act, [&]() {
+            return heavy_transmittance(F.m0_log2e, power_fraction_generic<N, float2>(F, z, w0), F.kind == kFrameGeneric);
+        });
     }
 };
 
