@@ -116,22 +116,10 @@ MB_HD float fdiv_fast(float a, float b) {
 #endif
 }
 MB_HD float frcp(float x) { return fdiv_fast(1.0f, x); }
-// the second operand where the first is NaN (a limit, never NaN); on the
-// device one instruction, where the comparison and select are two
-MB_HD float fmin_(float a, float b) {
-#if defined(__CUDA_ARCH__)
-    return fminf(a, b);
-#else
-    return a < b ? a : b;
-#endif
-}
-MB_HD float fmax_(float a, float b) {
-#if defined(__CUDA_ARCH__)
-    return fmaxf(a, b);
-#else
-    return a > b ? a : b;
-#endif
-}
+// the other operand where one is NaN; on the device one instruction, where a
+// comparison and select are two
+MB_HD float fmin_(float a, float b) { return fminf(a, b); }
+MB_HD float fmax_(float a, float b) { return fmaxf(a, b); }
 MB_HD float fclamp(float x, float lo, float hi) { return fmin_(fmax_(x, lo), hi); }
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -235,8 +223,12 @@ MB_HD bool lattice_range(const float o[3], const float d[3], const float lo[3], 
         float a = (lo[c] - o[c]) * inv, b = (hi[c] - o[c]) * inv;
         if (a > b) { float s = a; a = b; b = s; }
         float pad = (fabsf(o[c]) + fabsf(lo[c]) + fabsf(hi[c]) + 1.0f) * 3.814697265625e-06f * fabsf(inv);
-        t0 = fmax_(t0, a - pad);
-        t1 = fmin_(t1, b + pad);
+        // comparisons that let a NaN through (a direction that vanishes has no
+        // length to divide by): it refuses the ray below, where a minimum that
+        // drops it would leave all 2^22 lattice points to step through
+        const float ta = a - pad, tb = b + pad;
+        t0 = t0 > ta ? t0 : ta;
+        t1 = t1 < tb ? t1 : tb;
     }
     if (!(t1 >= t0)) return false;
     float inv_step = 1.0f / step;

@@ -145,7 +145,8 @@ __device__ __forceinline__ int skip_unit(const V& vol, int unit, const float o[3
         const float inv = 1.0f / d[c];
         const float tc = (face - o[c]) * inv;
         const float pad = (fabsf(o[c]) + fabsf(face) + 1.0f) * 3.814697265625e-06f * fabsf(inv);
-        t_exit = fmin_(t_exit, tc - pad);
+        const float te = tc - pad;
+        t_exit = t_exit < te ? t_exit : te;   // lets a NaN through: no skip then
     }
     const float kn = ceilf(t_exit / g.step - 0.5f) - 1.0f;
     if (!(kn > (float)(k + 1))) return k + 1;
