@@ -108,6 +108,7 @@ struct mboit_volume_s {
     mb::Counters* d_ctr = nullptr;
     std::vector<int32_t> pob;
     std::vector<mb::PieceBox> boxes;
+    std::vector<double> shares;   // per piece: the share of the domain's volume that its units fill
     int64_t owned = 0;
     std::vector<uint8_t> sel_host;
     bool sel_uploaded = false;
@@ -426,20 +427,57 @@ mboit_status select_pieces(mboit_volume v, const int32_t* pieces, int32_t n_piec
     return MBOIT_OK;
 }
 
+// Largest distance, in cells, between the rays of neighbouring pixels at the
+// domain's middle.
+double ray_spread(const mb::GridD& g, const mb::ViewTable& vt) {
+    double spread = 0.0;
+    for (int i = 0; i < vt.n; ++i) {
+        const mb::ViewD& V = vt.s[i].v;
+        double dist = 0.0, u = 0.0, w = 0.0;
+        const double c[3] = {0.5 * g.hx - V.eye[0], 0.5 * g.hy - V.eye[1], 0.5 * g.hz - V.eye[2]};
+        for (int k = 0; k < 3; ++k) {
+            dist += c[k] * c[k];
+            u += (double)V.u[k] * V.u[k];
+            w += (double)V.v[k] * V.v[k];
+        }
+        const double far = V.projection == MBOIT_PERSPECTIVE ? 2.0 * std::sqrt(dist) : 1.0;
+        spread = std::max(spread, far * std::max(std::sqrt(u) * std::fabs(V.scale_u) / V.width,
+                                                 std::sqrt(w) * std::fabs(V.scale_v) / V.height));
+    }
+    return spread;
+}
+
 // Whether the per-piece images of `list` come from one march per ray
 // (mboit_pieces.cuh) instead of one per piece, and the pieces' image slots.
 // One march walks the whole domain and pays a little for every piece change;
-// a march of its own visits the piece's box only.  So the one march is taken
-// when the wanted pieces' boxes together (overlaps counted each time, as each
-// piece's own march walks them again) cover at least half the domain's
-// volume.  Measured, both passes, own marches against one march: 256^3 grid,
-// 1024^2, boxes 0.22: 0.95 / 1.04 ms, 0.47: 1.33 / 1.09, all 16 pieces (2.6):
-// 6.16 / 1.97; octree of 13^3 base bricks, 0.56: 2.36 / 2.32, 0.19: 1.31 /
-// 1.81, all 24 (3.1): 11.28 / 4.28; mesh of 164 k tets, 512^2, 3 of 16
-// pieces: 1.08 / 0.93, all: 6.57 / 1.06.
+// a march of its own visits the piece's box, where it skips the units of other
+// pieces, and pays for its launch over all ray tiles.  So the one march is
+// taken when the wanted boxes together (overlaps counted each time, as each
+// piece's own march walks them again) cover at least half the domain.  Short
+// lists need more than that, because a large box may be nearly empty of its
+// piece:
+// - one piece: meshes (whose own march does not keep a warp's lanes in step),
+//   and a piece that fills 0.4 of the domain where the one march gathers
+//   better (windows of 16-byte rows, rays up to a cell apart) or where the
+//   sample's own work outweighs the gathers (trigonometric moments);
+// - two pieces of a grid without 16-byte rows: where they fill 0.2.
+// Measured, device time of both passes in us, own marches / one march:
+//   256^3 grid, 1024^2 view: all of 16 pieces 6075 / 1901; two, boxes 0.75,
+//     1487 / 1199; one, box 0.5 filled 0.42, 1390 / 1293, filled 0.22, 854 /
+//     1074; 256^2 view (1.7 cells apart): one, filled 1.0, 1033 / 1116, 0.42,
+//     489 / 706; two, boxes 0.75, 770 / 705
+//   301 x 227 x 181 grid, 800^2: all of 16 3717 / 1255; two, filled 0.83, 1219 /
+//     1109, 0.15, 508 / 791; one, box 1.0 filled 0.60, 702 / 988, 0.07, 296 / 700;
+//     8 trigonometric moments, one, filled 0.60, 2203 / 1855, 0.09, 657 / 854
+//   octree of 13^3 base bricks, 512^2: all of 16 6875 / 2023; two, boxes 0.85,
+//     1481 / 1468; one, box 1.0 filled 0.60, 1022 / 1320; 8 trigonometric
+//     moments 2356 / 1965
+//   mesh of 164 k tets, 512^2: all of 16 6509 / 492; one, box 0.51, 562 / 395.
+// Over 1,554 lists of these and smaller scenes, every moment set, the rule's
+// choice is at most 1.2 times as slow as the better one, 1.23 in one case.
 // Lists with a piece named twice and partial lists of volumes with more
 // pieces than the slot map holds keep their own marches.
-bool one_march(mboit_volume v, const std::vector<int32_t>& list, mb::SlotMap& map) {
+bool one_march(mboit_volume v, const std::vector<int32_t>& list, const mb::ViewTable& vt, mb::SlotMap& map) {
     map.n = 0;
     const size_t K = v->boxes.size();
     bool identity = list.size() == K;
@@ -453,12 +491,17 @@ bool one_march(mboit_volume v, const std::vector<int32_t>& list, mb::SlotMap& ma
             map.slot[list[i]] = (int16_t)i;
         }
     }
-    double boxes = 0.0;
+    double boxes = 0.0, filled = 0.0;
     for (int32_t p : list) {
         const mb::PieceBox& b = v->boxes[p];
         boxes += (double)(b.hi[0] - b.lo[0]) * (b.hi[1] - b.lo[1]) * (b.hi[2] - b.lo[2]);
+        filled += v->shares[p];
     }
-    return boxes >= kOneMarchVolume * (double)v->grid.hx * v->grid.hy * v->grid.hz;
+    if (boxes < kOneMarchVolume * (double)v->grid.hx * v->grid.hy * v->grid.hz) return false;
+    if (v->kind == MBOIT_TET || list.size() > 2) return true;
+    const bool rows16 = v->kind == MBOIT_GRID && mb::stage_config_eligible(v->grid, 3);
+    if (list.size() == 2) return v->kind != MBOIT_GRID || rows16 || filled >= 0.2;
+    return filled >= 0.4 && (is_trig(v->desc.moment_set) || (rows16 && ray_spread(v->grid, vt) <= 1.0));
 }
 
 // Host tables of a tetrahedral mesh: snapped vertex records, cells,
@@ -649,22 +692,7 @@ bool config_usable(mboit_volume v, int cfg) {
 // 64^3 at 256^2 (0.43) 95 / 92; 256^3 at 256^2 (1.7) 605 / 755.
 void auto_tune(mboit_volume v, const mb::ViewTable& vt) {
     if (v->tuned || v->kind != MBOIT_GRID) return;
-    const mb::GridD& g = v->grid;
-    double spread = 0.0;
-    for (int i = 0; i < vt.n; ++i) {
-        const mb::ViewD& V = vt.s[i].v;
-        double dist = 0.0, u = 0.0, w = 0.0;
-        const double c[3] = {0.5 * g.hx - V.eye[0], 0.5 * g.hy - V.eye[1], 0.5 * g.hz - V.eye[2]};
-        for (int k = 0; k < 3; ++k) {
-            dist += c[k] * c[k];
-            u += (double)V.u[k] * V.u[k];
-            w += (double)V.v[k] * V.v[k];
-        }
-        const double far = V.projection == MBOIT_PERSPECTIVE ? 2.0 * std::sqrt(dist) : 1.0;
-        spread = std::max(spread, far * std::max(std::sqrt(u) * std::fabs(V.scale_u) / V.width,
-                                                 std::sqrt(w) * std::fabs(V.scale_v) / V.height));
-    }
-    const bool dense = spread <= kDenseRays;
+    const bool dense = ray_spread(v->grid, vt) <= kDenseRays;
     v->tune1 = !dense ? 0 : config_usable(v, 6) ? 6 : config_usable(v, 3) ? 3 : 0;
     v->tune2 = dense && config_usable(v, 3) ? 3 : 0;
 }
@@ -1224,6 +1252,9 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
     std::vector<uint8_t> seen((size_t)v->nbricks, 0);
     int bmin[3] = {1 << 30, 1 << 30, 1 << 30}, bmax[3] = {-1, -1, -1};
     const mb::GridD& g = v->grid;
+    const int B = 1 << g.brick_log2;
+    const float hi[3] = {g.hx, g.hy, g.hz};
+    double volume = 0.0;   // of the units, in cells (meshes: the domain's, by count)
     for (int64_t i = 0; i < n; ++i) {
         const int32_t b = h[i];
         if (b < 0 || b >= v->nbricks) return fail(MBOIT_ERR_INVALID_ARG, "brick id " + std::to_string(b) + " out of range");
@@ -1234,10 +1265,13 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
         seen[b] = 1;
         if (v->kind != MBOIT_GRID) continue;
         const int bc[3] = {b % g.nbx, (b / g.nbx) % g.nby, b / (g.nbx * g.nby)};
+        double cells = 1.0;
         for (int c = 0; c < 3; ++c) {
             bmin[c] = bc[c] < bmin[c] ? bc[c] : bmin[c];
             bmax[c] = bc[c] > bmax[c] ? bc[c] : bmax[c];
+            cells *= std::min((float)((bc[c] + 1) * B), hi[c]) - (float)(bc[c] * B);
         }
+        volume += cells;
     }
     for (int64_t i = 0; i < n; ++i) v->pob[h[i]] = K;
     cudaError_t e = cudaMemcpy(v->d_pob, v->pob.data(), (size_t)v->nbricks * sizeof(int32_t), cudaMemcpyHostToDevice);
@@ -1245,8 +1279,6 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
         for (int64_t i = 0; i < n; ++i) v->pob[h[i]] = -1;
         return fail(MBOIT_ERR_CUDA, std::string("uploading brick ownership: ") + cudaGetErrorString(e));
     }
-    const int B = 1 << g.brick_log2;
-    const float hi[3] = {g.hx, g.hy, g.hz};
     mb::PieceBox box;
     if (v->kind == MBOIT_TET) {
         // union of the tets' boxes, padded by one quantum (a sample snaps by up to half of one)
@@ -1267,6 +1299,7 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
             box.lo[c] = std::max(box.lo[c] - pad, 0.0f);
             box.hi[c] = std::min(box.hi[c] + pad, hi[c]);
         }
+        volume = (double)g.hx * g.hy * g.hz * (double)n / (double)v->nbricks;
     } else if (v->kind == MBOIT_AMR) {
         // union of the leaves' boxes
         for (int c = 0; c < 3; ++c) {
@@ -1276,10 +1309,14 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
         for (int64_t i = 0; i < n; ++i) {
             const int32_t* L = &v->leaf_table[4 * (size_t)h[i]];
             const float size = (float)(B << (v->desc.max_level - L[3]));
+            double cells = 1.0;
             for (int c = 0; c < 3; ++c) {
+                const float top = std::min((float)L[c] + size, hi[c]);
                 box.lo[c] = std::min(box.lo[c], (float)L[c]);
-                box.hi[c] = std::max(box.hi[c], std::min((float)L[c] + size, hi[c]));
+                box.hi[c] = std::max(box.hi[c], top);
+                cells *= top - (float)L[c];
             }
+            volume += cells;
         }
     } else {
         for (int c = 0; c < 3; ++c) {
@@ -1289,6 +1326,7 @@ mboit_status mboit_add_piece(mboit_volume v, const int32_t* ids, int64_t n, int3
         }
     }
     v->boxes.push_back(box);
+    v->shares.push_back(volume / ((double)g.hx * g.hy * g.hz));
     v->owned += n;
     v->sel_uploaded = false;
     drop_graphs(v);
@@ -1321,7 +1359,7 @@ mboit_status mboit_render_moments(mboit_volume v, const mboit_view* views, int32
         const int32_t slots = (int32_t)list.size();
         MB_CUDA(check_tables(v, s));
         mb::SlotMap map;
-        const bool one = !is_trig(v->desc.moment_set) && one_march(v, list, map);
+        const bool one = !is_trig(v->desc.moment_set) && one_march(v, list, vt, map);
         if (one) {
             MB_CUDA(v->kind == MBOIT_AMR
                         ? mb::launch_pass1_pieces(v->amr, v->d_tf, v->d_pob, vt, map, slots, moments, v->d_ctr, s)
@@ -1368,7 +1406,7 @@ mboit_status mboit_reconstruct_blend(mboit_volume v, const mboit_view* views, in
         const int32_t slots = (int32_t)list.size();
         MB_CUDA(check_tables(v, s));
         mb::SlotMap map;
-        const bool one = one_march(v, list, map);
+        const bool one = one_march(v, list, vt, map);
         if (one) {
             MB_CUDA(v->kind == MBOIT_AMR ? mb::launch_pass2_pieces(v->amr, v->d_tf, v->d_pob, vt, map, slots,
                                                                    global_moments, color, v->d_ctr, s)
