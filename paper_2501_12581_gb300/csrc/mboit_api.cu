@@ -687,9 +687,15 @@ bool config_usable(mboit_volume v, int cfg) {
 // it, else 3) for pass 1 and 3 for pass 2 where neighbouring rays lie within
 // kDenseRays cells of each other at the domain's middle, so that a warp's window
 // spans many lattice steps; else 0, whose small windows fall back to direct
-// loads soonest.  Measured, one-launch frames in configurations 0 / 6: 256^3
-// at 1024^2 (0.42 cells) 1115 / 965 us, 256 x 96 x 320 at 900 x 700 434 / 330,
-// 64^3 at 256^2 (0.43) 95 / 92; 256^3 at 256^2 (1.7) 605 / 755.
+// loads soonest.  The line is pass 2's: split pass 2 in configurations 0 / 3
+// (us), 256^3 grid, rays 0.4 cells apart 949 / 829, 0.6 578 / 500, 0.75 492 /
+// 497, 0.8 495 / 535, 0.9 509 / 596; 512^3, 0.6 3925 / 3077, 0.75 2956 / 2699,
+// 0.8 2779 / 2861; 128^3, 0.4 184 / 190, 0.75 185 / 169, 0.9 189 / 182; 64^3, 0.2
+// 98 / 103.  Pass 1 in configuration 6 wins to about 1.2 cells (256^3, two-launch
+// frame in configurations 0 / 6 and 3: 0.75 cells 665 / 467, 1.2 613 / 481, 1.5
+// 640 / 653, 2.0 722 / 787).  6 and 8 power and trigonometric moments
+// (configuration 3 in both passes): at 0.75 cells 4 to 36 % faster than in 0, at
+// 1.0 between 9 % slower and 14 % faster.
 void auto_tune(mboit_volume v, const mb::ViewTable& vt) {
     if (v->tuned || v->kind != MBOIT_GRID) return;
     const bool dense = ray_spread(v->grid, vt) <= kDenseRays;

@@ -352,17 +352,16 @@ __device__ __forceinline__ bool march_fused(const GridD& g, const uint8_t* __res
 }
 
 
-// Pass 2 marching the field, two points at a time in a warp whose lanes with
-// samples all may (pairs()): the same bits.
+// Pass 2 marching the field (no TMA windows there), two points at a time in a
+// warp whose lanes with samples all may (pairs()): the same bits.
 template <class Cfg, bool kSel, class Body>
 __device__ __forceinline__ bool blend_fused(const GridD& g, const uint8_t* __restrict__ sel, float* __restrict__ win,
-                                            const float o[3], const float d[3], int k0, int k1, Body& body,
-                                            TmaWin* tma = nullptr) {
+                                            const float o[3], const float d[3], int k0, int k1, Body& body) {
     if (__all_sync(0xffffffffu, k0 > k1 || body.pairs())) {
         PairBlend<Body> pb{body};
-        return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, pb, NoStore{}, tma);
+        return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, pb);
     }
-    return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body, NoStore{}, tma);
+    return march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
 }
 
 // The same for a tile whose rows found no room in the sample cache, as a call:
@@ -461,7 +460,7 @@ __global__ void __launch_bounds__(256) k_pass2_fused(const __grid_constant__ Gri
             // this rare march takes no registers from the loop over the rows
             march_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
         } else {
-            blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);   // pass 2 has no TMA windows
+            blend_fused<Cfg, kSel>(g, sel, win, o, d, k0, k1, body);
         }
         if (valid) {
             float4* out = reinterpret_cast<float4*>(color + S.color_off) + pix;

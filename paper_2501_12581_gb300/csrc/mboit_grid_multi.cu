@@ -7,8 +7,9 @@
 // volumes share one transfer function (staged once per CTA in shared
 // memory); their fields, domains, sampling steps and moment parameters are
 // their own, read from the GridTable kernel parameter by the view's index.
-// The per-tile code is the single-volume frame's (march_fused, blend_rows,
-// march_fused), so every pixel equals its volume's own frame bit for bit.
+// The per-tile code is the single-volume frame's (march_fused in pass 1 and for
+// tiles whose rows found no room, blend_rows in pass 2), so every pixel equals
+// its volume's own frame bit for bit.
 #include "mboit_grid.cuh"
 
 namespace mb {

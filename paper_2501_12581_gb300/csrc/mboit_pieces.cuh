@@ -19,9 +19,13 @@
 // piece changes (16 to 20 bytes out and in per change, mostly L2 hits).  256^3
 // grid in 16 pieces, 1024^2 view (193 M samples), passes 1 and 2 with the
 // clearing of the images: 2.85 + 3.31 ms as own marches, 0.81 + 1.16 ms as
-// one.  What bounds it is what bounds the fused passes (issue and the windows'
-// shared-memory reads), with the brick of each sample and the piece changes
-// on top.
+// one.  What bounds it is issue (72 % of the slots in pass 1, 81 % in pass 2, with
+// the windows' shared-memory reads at 67 and 58 % of the L1 pipe), one point at
+// a time with the brick of each sample: 103 and 170 warp instructions per
+// 32 samples, where the frame's passes take 72 and 56 (two points at a time,
+// pass 2 from the sample cache).  The images' traffic does not show: DRAM 2 %,
+// 92 % of the L2 reads hit.  Lists of one or two pieces may be better off with
+// marches of their own (one_march).
 #pragma once
 #include "mboit_grid.cuh"
 #include "mboit_pieces.h"

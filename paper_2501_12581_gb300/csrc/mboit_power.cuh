@@ -18,10 +18,17 @@
 //     1 / K(x_i, x_i) of the roots in front,
 //     A = w0 / K(x0, x0) + sum_{x_i < x0} 1 / K(x_i, x_i),
 //     or, where fewer roots lie behind, 1 less their weights (front_weight).
-// Every weight is a sum of positive terms, so no cancellation enters A.  A
-// pixel whose Hankel matrix is numerically singular (a pivot below 1e-12 of
-// its diagonal entry: no bias and at most n absorbers) falls back to the
-// four-moment frame, which handles one- and two-atom measures exactly.
+// Every weight is the reciprocal of a sum of positive terms, so no cancellation
+// enters a weight.  Taking A as 1 less the weights behind adds a rounding of 1:
+// nothing to T = e^(-b0 A), which takes A's absolute error, but small A lose
+// relative accuracy.  Root mean square error of A against 64 bits over the host
+// check's rays, all weights in front / the smaller side: 6 power moments 8.6e-7
+// / 7.1e-7, 8 2.0e-6 / 1.8e-6, 6 trigonometric 2.0e-7 / 1.1e-7, 8 3.0e-7 / 2.5e-7;
+// the largest error is the same or smaller (relative, for A above 0.01: 6 and 8
+// trigonometric moments 3.0e-6 and 8.7e-6 / 2.1e-5 and 1.4e-5).  A pixel whose
+// Hankel matrix is numerically singular (a pivot below 1e-12 of its diagonal
+// entry: no bias and at most n absorbers) falls back to the four-moment frame,
+// which handles one- and two-atom measures exactly.
 #pragma once
 #include "mboit_trig.cuh"
 

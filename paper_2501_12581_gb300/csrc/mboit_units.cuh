@@ -358,8 +358,8 @@ __device__ __forceinline__ bool outside(long long D, int nx, int ny, int nz) {
 // edges below 2^15 quanta, so the stored normals fit in 32 bits and three
 // faces are three 32 x 32 -> 64-bit multiply-adds each, the fourth the
 // volume's remainder.  (From the corners a face cost six products, twelve
-// differences and those three multiply-adds; the record has the size the
-// corners had.)
+// differences and those three multiply-adds.  The record has the corners' 64
+// bytes; the corner values, which those held too, are 16 bytes beside it.)
 __device__ __forceinline__ void tet_volumes(const int4 v[4], const int q[3], long long D[4]) {
     const int dx = q[0] - v[0].x, dy = q[1] - v[0].y, dz = q[2] - v[0].z;
 #pragma unroll
@@ -553,8 +553,8 @@ __device__ __forceinline__ bool piece_sample(const TetT<kNarrow>& m, const int32
 // (One loop of tet tests, each lane on its own row, sampled a few lanes at a
 // time.)  1.3 M tets, 1024^2 view (48 M samples): 2.11 ms of pass 1 with tests
 // from the corners in one loop, 1.36 with stored normals in lockstep, 0.95
-// with the walk by the largest volume.  The walk's loads (one 80-byte
-// visit per face crossed, about 1.8 per sample) and the lanes that wait for the
+// with the short loop over whole volumes.  The walk's loads (one 80-byte
+// visit per face crossed, about 1.7 per sample) and the lanes that wait for the
 // longest walk of their row bound it.  Every point has one owner, so the order
 // in which faces are crossed does not matter.  `store` gets every lattice point's value (NaN: not
 // sampled).  With zrows (a warp's DepthRows) the moments take the rows' shared
@@ -591,8 +591,12 @@ __device__ __forceinline__ void march_unit(const TetT<kNarrow>& m, const uint8_t
             int skip = -1, f = 0, steps = 0;
             if constexpr (kNarrow) {
                 // the faces that the point lies strictly outside of, the
-                // largest volume (its high word) first: shorter walks than
-                // the first face found, and no test for points on a face.
+                // largest volume (its high word) first.  Most of what this
+                // loop gained (1.36 -> 0.95 ms of pass 1, see above) is that
+                // it picks the face without a rotation and has no test for
+                // points on a face; the largest volume instead of the first
+                // one found is 2.65 tets tested per point against 2.73 (24^3
+                // jittered cells, half-cell steps) and 0.93 against 1.00 ms.
                 // The full test below then runs once, the lanes together
                 // (skipping it where no volume is 0 parts them: 1.24 ms a
                 // frame against 1.13)
@@ -1110,14 +1114,7 @@ __global__ void __launch_bounds__(256, MS == 0 ? MinBlocks<V, 1>::value : 2) k_p
         int k0, k1;
         ray_range(g, S.v, valid, px, py, o, d, k0, k1);
         auto body = make_moment_body<MS>(s_sig, g, S.v);
-        if constexpr (std::is_same<V, AmrD>::value) {
-            if constexpr (kCache) {
-                RowStore st{tile_rows(cache, ctr, tile, k0, k1)};
-                march_unit<kSel>(a, sel, o, d, k0, k1, body, st, zrows);
-            } else {
-                march_unit<kSel>(a, sel, o, d, k0, k1, body, NoStore{}, zrows);
-            }
-        } else if constexpr (kCache) {
+        if constexpr (kCache) {
             RowStore st{tile_rows(cache, ctr, tile, k0, k1)};
             march_unit<kSel>(a, sel, o, d, k0, k1, body, st, zrows);
         } else {
