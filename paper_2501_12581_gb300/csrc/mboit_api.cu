@@ -1507,11 +1507,10 @@ mboit_status mboit_render_frame(mboit_volume v, const mboit_view* views, int32_t
         cudaStream_t cs = v->cap_stream;
         MB_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = mb::clear_frame_counters(v->d_ctr, cs);
-        // external record nodes: the events are recorded each time the graph runs;
-        // the table check belongs to pass 1's time
-        if (e == cudaSuccess) e = cudaEventRecordWithFlags(v->frame_ev[0], cs, cudaEventRecordExternal);
         if (e == cudaSuccess) e = check_tables(v, cs);
         tc.cleared = 1;
+        // external record nodes: the events are recorded each time the graph runs
+        if (e == cudaSuccess) e = cudaEventRecordWithFlags(v->frame_ev[0], cs, cudaEventRecordExternal);
         if (v->frame_launches == 1) {
             if (e == cudaSuccess) e = frame_batched(v, mask, vt, moments_scratch, rgba, cs, v->tune1, tc);
             if (e == cudaSuccess) e = cudaEventRecordWithFlags(v->frame_ev[1], cs, cudaEventRecordExternal);
