@@ -222,8 +222,10 @@ typedef struct {
                                  * set up in FP64: a variance or Schur complement of the biased Hankel matrix
                                  * within 1e-4 of b2 or b4 (near-singular); every other pixel is set up in
                                  * float-float FP32 arithmetic */
-    float frame_pass1_ms;       /* device time of pass 1 in the last mboit_render_frame (CUDA events
-                                 * recorded in its graph); -1 before the first frame */
+    float frame_pass1_ms;       /* device time of pass 1's kernel in the last mboit_render_frame (CUDA events
+                                 * recorded in its graph); -1 before the first frame.  Neither time holds
+                                 * what a frame does once before its first event: the clearing of its
+                                 * counters and the check of an octree's or mesh's index tables */
     float frame_pass2_ms;       /* the same for pass 2 */
     int32_t packet;             /* mboit_packet in use (see mboit_set_packet) */
     int32_t frame_launches;     /* kernel launches of mboit_render_frame (see mboit_set_frame_launches);
